@@ -8,10 +8,9 @@
 
 namespace atspeed {
 
-// h_out/x rows: x[t] = bf16(rmsnorm(h[t]) * g); with `tokens`, h[t] = embed[tokens[t]] first.
-cudaError_t rmsnorm_launch(const float* h, const int* tokens, const __nv_bfloat16* embed, float* h_out,
-                           const __nv_bfloat16* g, int T, int d, float eps, __nv_bfloat16* x, int ldx,
-                           cudaStream_t st, bool pdl);
+// x[t] = bf16(rmsnorm(h[t]) * g), h [T][d] fp32, x [T][ldx]
+cudaError_t rmsnorm_launch(const float* h, const __nv_bfloat16* g, int T, int d, float eps, __nv_bfloat16* x, int ldx,
+                           cudaStream_t st);
 
 // Layer 0's rows with the first norm folded into the QKV GEMM: h[t] = embed[tokens[t]],
 // xg[t] = bf16(g * h[t]), ssq[mt * ld + t] = partial sums of squares of h[t] per 128-row tile.

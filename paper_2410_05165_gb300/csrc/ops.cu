@@ -130,8 +130,8 @@ atspeed_status atspeed_op_gemm_swiglu(atspeed_stream stream, const void* d_W, co
 atspeed_status atspeed_op_rmsnorm(atspeed_stream stream, const float* d_h, const void* d_g, int T, int d, float eps,
                                   void* d_x, int ldx) {
   if (!d_h || !d_g || !d_x || T <= 0 || d <= 0 || ldx < d) return ATSPEED_E_ARG;
-  const cudaError_t e = rmsnorm_launch(d_h, nullptr, nullptr, nullptr, static_cast<const __nv_bfloat16*>(d_g), T, d,
-                                       eps, static_cast<__nv_bfloat16*>(d_x), ldx, (cudaStream_t)stream, false);
+  const cudaError_t e = rmsnorm_launch(d_h, static_cast<const __nv_bfloat16*>(d_g), T, d, eps,
+                                       static_cast<__nv_bfloat16*>(d_x), ldx, (cudaStream_t)stream);
   return e == cudaSuccess ? ATSPEED_OK : ATSPEED_E_CUDA;
 }
 
