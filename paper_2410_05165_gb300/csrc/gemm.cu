@@ -381,17 +381,41 @@ cudaError_t launch_bn(EpiKind e, const CUtensorMap& ma, const CUtensorMap& mb, c
   return cudaErrorInvalidValue;
 }
 
-__global__ void lse_combine_kernel(const float2* part, int ld, int m_tiles, int T, float* lse) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T) return;
-  float mx = -INFINITY;
-  for (int m = 0; m < m_tiles; ++m) mx = fmaxf(mx, part[(size_t)m * ld + t].x);
-  float s = 0.f;
-  if (mx != -INFINITY)
-    for (int m = 0; m < m_tiles; ++m) {
-      const float2 v = part[(size_t)m * ld + t];
-      if (v.x != -INFINITY) s += v.y * expf(v.x - mx);
+// Log-sum-exp of each token's row from its m_tiles partials (max, sum of exp): 32 tokens per CTA, warp w
+// combines the tiles w, w + LSE_WARPS, ... of its 32 tokens (one coalesced load per tile), then the
+// warps' results are combined in warp order, so a token's value depends on m_tiles alone.
+// Latency-bound: one thread per token and two passes over 258 tiles took 40.7 us for 960 tokens and 29.7
+// us for 4; sixteen warps per 32 tokens and one pass with eight loads in flight: 7.0 us.
+constexpr int LSE_WARPS = 16;
+__global__ void __launch_bounds__(32 * LSE_WARPS) lse_combine_kernel(const float2* part, int ld, int m_tiles, int T,
+                                                                     float* lse) {
+  __shared__ float2 red[LSE_WARPS][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, t = blockIdx.x * 32 + lane;
+  // s counts in units of exp(mx); an empty partial is (-inf, 0)
+  float mx = -INFINITY, s = 0.f;
+  auto add = [&](float2 v) {
+    const float m2 = fmaxf(mx, v.x);
+    if (m2 == -INFINITY) return;
+    s = s * expf(mx - m2) + v.y * expf(v.x - m2);
+    mx = m2;
+  };
+  for (int m0 = w; m0 < m_tiles; m0 += 8 * LSE_WARPS) {
+    float2 v[8];   // eight loads in flight
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int m = m0 + i * LSE_WARPS;
+      v[i] = t < T && m < m_tiles ? part[(size_t)m * ld + t] : make_float2(-INFINITY, 0.f);
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) add(v[i]);
+  }
+  red[w][lane] = make_float2(mx, s);
+  __syncthreads();
+  if (w != 0 || t >= T) return;
+  mx = -INFINITY;
+  s = 0.f;
+#pragma unroll
+  for (int i = 0; i < LSE_WARPS; ++i) add(red[i][lane]);
   lse[t] = mx + logf(s);
 }
 
@@ -399,7 +423,7 @@ __global__ void lse_combine_kernel(const float2* part, int ld, int m_tiles, int 
 
 cudaError_t lse_combine_launch(const float2* part, int ld, int m_tiles, int T, float* lse, cudaStream_t st) {
   if (T <= 0) return cudaSuccess;
-  lse_combine_kernel<<<(T + 127) / 128, 128, 0, st>>>(part, ld, m_tiles, T, lse);
+  lse_combine_kernel<<<(T + 31) / 32, 32 * LSE_WARPS, 0, st>>>(part, ld, m_tiles, T, lse);
   return cudaGetLastError();
 }
 

@@ -63,7 +63,7 @@ struct GemmScratch {
 };
 
 // log-sum-exp of each token's whole row from the EPI_LSE partials of m_tiles row tiles, combined in
-// tile order: lse[t] = log sum_m s_m exp(max_m - max) + max.
+// a fixed order: lse[t] = log sum_m s_m exp(max_m - max) + max.
 cudaError_t lse_combine_launch(const float2* part, int ld, int m_tiles, int T, float* lse, cudaStream_t st);
 
 // Bytes of split-K workspace / counters needed for a grid of `grid` CTAs.
