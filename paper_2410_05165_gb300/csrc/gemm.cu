@@ -440,37 +440,40 @@ int gemm_grid_size(int device) {
   return sms > 0 ? sms : 1;
 }
 
-cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaStream_t stream, bool pdl,
-                        char* eb, size_t el) {
+cudaError_t gemm_check(const GemmArgs& a, int max_tiles, char* eb, size_t el) {
   if (a.K <= 0 || a.K % BK != 0 || a.K / BK > 256 || a.M <= 0 || a.T <= 0) {
     snprintf(eb, el, "gemm: bad shape M=%d K=%d T=%d", a.M, a.K, a.T);
     return cudaErrorInvalidValue;
   }
+  const int BN = a.T <= 128 ? 128 : 256, n_tiles = (a.T + BN - 1) / BN;
+  if (a.X_rows < n_tiles * BN) {
+    snprintf(eb, el, "gemm: X has %d rows, needs %d", a.X_rows, n_tiles * BN);
+    return cudaErrorInvalidValue;
+  }
+  if (a.epi == EPI_SWIGLU && a.M % 128 != 0) {
+    snprintf(eb, el, "gemm: SwiGLU needs 2*d_ffn %% 128 == 0 (M=%d)", a.M);
+    return cudaErrorInvalidValue;
+  }
+  const long long tiles = ((long long)a.M + BM - 1) / BM * n_tiles;
+  if (tiles > max_tiles) {
+    snprintf(eb, el, "gemm: %lld tiles exceed the counter table (%d)", tiles, max_tiles);
+    return cudaErrorInvalidValue;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaStream_t stream, bool pdl,
+                        char* eb, size_t el) {
+  const cudaError_t ce = gemm_check(a, s.max_tiles, eb, el);
+  if (ce != cudaSuccess) return ce;
   const int BN = a.T <= 128 ? 128 : 256;
   KParams kp;
   kp.a = a;
   kp.n_tiles = (a.T + BN - 1) / BN;
-  if (a.X_rows < kp.n_tiles * BN) {
-    snprintf(eb, el, "gemm: X has %d rows, needs %d", a.X_rows, kp.n_tiles * BN);
-    return cudaErrorInvalidValue;
-  }
-  if (a.epi == EPI_SWIGLU) {
-    if (a.M % 128 != 0) {
-      snprintf(eb, el, "gemm: SwiGLU needs 2*d_ffn %% 128 == 0 (M=%d)", a.M);
-      return cudaErrorInvalidValue;
-    }
-    kp.m_tiles = a.M / 128;
-    kp.up_row0 = a.M / 2;
-  } else {
-    kp.m_tiles = (a.M + BM - 1) / BM;
-    kp.up_row0 = 0;
-  }
+  kp.m_tiles = (a.M + BM - 1) / BM;
+  kp.up_row0 = a.epi == EPI_SWIGLU ? a.M / 2 : 0;
   kp.kb = a.K / BK;
   const long long tiles = (long long)kp.m_tiles * kp.n_tiles;
-  if (tiles > s.max_tiles) {
-    snprintf(eb, el, "gemm: %lld tiles exceed the counter table (%d)", tiles, s.max_tiles);
-    return cudaErrorInvalidValue;
-  }
   kp.G = gemm_work_ctas(tiles, kp.kb, grid);
   kp.w = work_split((int)tiles, kp.kb, kp.G);
   if (s.ws_bytes < gemm_ws_bytes(kp.G)) {

@@ -79,8 +79,17 @@ bool gemm_make_map(CUtensorMap* m, const void* base, int inner, int rows, int bo
 // address or row pitch breaks the TMA alignment rules); cudaErrorInvalidValue means a bad shape.
 constexpr cudaError_t kGemmMapError = cudaErrorInvalidDevicePointer;
 
+// The shapes that the GEMMs run: cudaErrorInvalidValue (with a message) for the others.
+cudaError_t gemm_check(const GemmArgs& a, int max_tiles, char* errbuf, size_t errlen);
+
 // Encodes the tensor maps and launches.  `pdl` enables programmatic dependent launch.
 cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaStream_t stream, bool pdl,
                         char* errbuf, size_t errlen);
+
+// The operators' GEMM with few output tiles (gemm_cluster.cu): EPI_F32, EPI_RESID and EPI_SWIGLU, no
+// workspace.  gemm_cluster_fits: whether it is the kernel for these sizes on a GPU of `sms` SMs.
+bool gemm_cluster_fits(const GemmArgs& a, int sms);
+cudaError_t gemm_cluster_launch(const GemmArgs& a, unsigned int* err, int sms, cudaStream_t stream, char* errbuf,
+                                size_t errlen);
 
 }  // namespace atspeed

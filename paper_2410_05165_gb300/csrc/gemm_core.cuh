@@ -302,6 +302,12 @@ __device__ __forceinline__ void ws_reduce_resnorm_half(const GemmArgs& a, const 
   resnorm_store<16, SR>(a, st, m_tile, tok0, j0, nv, ep_tid);
 }
 
+// silu(g) * u, silu(g) = g / (1 + e^-g), with the hardware exponential and an approximate divide (a few
+// ulp, far below the bf16 rounding of the product; for g -> -inf the divisor overflows to inf and the
+// quotient is -0); the IEEE expf and divide made the epilogue's loop latency-bound (about 2 us per
+// 32-token chunk)
+__device__ __forceinline__ float swiglu(float g, float u) { return __fdividef(g, 1.0f + __expf(-g)) * u; }
+
 // st: staging [32 tokens][128 rows] fp32 of one chunk; 128 threads (ep_tid) write the outputs.
 // tpos / tkvr: the n-tile's token tables (EPI_QKV only); trs: the n-tile's norm scales (EPI_QKV /
 // EPI_SWIGLU when the input rows are g * h, else null).
@@ -380,10 +386,7 @@ __device__ __forceinline__ void epi_chunk(const GemmArgs& a, const float* st, in
     }
   } else if constexpr (EPI == EPI_SWIGLU) {
     // thread owns features 2f, 2f + 1 of the tile (one 4-byte store per token) and tokens
-    // (ep_tid >> 5) + 4k.  silu(g) = g / (1 + e^-g) with the hardware exponential and an
-    // approximate divide (a few ulp, far below the bf16 rounding of the product; for g -> -inf the
-    // divisor overflows to inf and the quotient is -0); the IEEE expf and divide made this loop
-    // latency-bound (about 2 us per 32-token chunk)
+    // (ep_tid >> 5) + 4k
     const int f = ep_tid & 31, n0 = ep_tid >> 5;
     __nv_bfloat16* out = a.out_bf16 + m_tile * 64 + 2 * f;
     const int T = a.T;
@@ -406,9 +409,8 @@ __device__ __forceinline__ void epi_chunk(const GemmArgs& a, const float* st, in
     for (int k = 0; k < 8; ++k) {
       const int tok = tok0 + n0 + 4 * k;
       if (tok < T) {
-        const float y0 = __fdividef(gv[k].x, 1.0f + __expf(-gv[k].x)) * uv[k].x;
-        const float y1 = __fdividef(gv[k].y, 1.0f + __expf(-gv[k].y)) * uv[k].y;
-        *reinterpret_cast<__nv_bfloat162*>(out + (size_t)tok * ldo) = __floats2bfloat162_rn(y0, y1);
+        *reinterpret_cast<__nv_bfloat162*>(out + (size_t)tok * ldo) =
+            __floats2bfloat162_rn(swiglu(gv[k].x, uv[k].x), swiglu(gv[k].y, uv[k].y));
       }
     }
   } else if constexpr (EPI == EPI_LSE) {

@@ -49,7 +49,10 @@ atspeed_status gemm_status(cudaError_t e) {
 atspeed_status run_gemm(cudaStream_t st, const GemmArgs& a, void* ws) {
   if (!ws) return ATSPEED_E_ARG;
   char eb[256];
-  return gemm_status(gemm_launch(a, scratch_from(ws), current_grid(), st, false, eb, sizeof eb));
+  const int grid = current_grid();
+  const GemmScratch s = scratch_from(ws);
+  if (gemm_cluster_fits(a, grid)) return gemm_status(gemm_cluster_launch(a, s.err, grid, st, eb, sizeof eb));
+  return gemm_status(gemm_launch(a, s, grid, st, false, eb, sizeof eb));
 }
 
 // ---------------------------------------------------------------------------------------------
