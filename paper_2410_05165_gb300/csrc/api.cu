@@ -428,10 +428,10 @@ void alloc_model(atspeed_ctx* c, ModelRt& m) {
   const int nmaps = fwd_map_count(m.layers);
   std::vector<CUtensorMap> hm(nmaps);
   for (int l = 0; l < m.layers; ++l) {
-    const bool ok = gemm_make_map(&hm[l * 4 + 0], m.wqkv[l], m.d, 3 * m.d, 64, eb, sizeof eb) &&
-                    gemm_make_map(&hm[l * 4 + 1], m.wo[l], m.d, m.d, 64, eb, sizeof eb) &&
-                    gemm_make_map(&hm[l * 4 + 2], m.wgate_up[l], m.d, 2 * m.ffn, 64, eb, sizeof eb) &&
-                    gemm_make_map(&hm[l * 4 + 3], m.wdown[l], m.ffn, m.d, 64, eb, sizeof eb);
+    const bool ok = gemm_make_map(&hm[l * 4 + 0], m.wqkv[l], m.d, 3 * m.d, 128, eb, sizeof eb) &&
+                    gemm_make_map(&hm[l * 4 + 1], m.wo[l], m.d, m.d, 128, eb, sizeof eb) &&
+                    gemm_make_map_pairs(&hm[l * 4 + 2], m.wgate_up[l], m.d, m.ffn, eb, sizeof eb) &&
+                    gemm_make_map(&hm[l * 4 + 3], m.wdown[l], m.ffn, m.d, 128, eb, sizeof eb);
     if (!ok) {
       set_err(c, "%s", eb);
       throw Fail{ATSPEED_E_CUDA};
@@ -440,7 +440,7 @@ void alloc_model(atspeed_ctx* c, ModelRt& m) {
     hm[4 * m.layers + 2 * l + 1] = m.mv[l];
   }
   const int L6 = 6 * m.layers;
-  bool ok = gemm_make_map(&hm[L6], m.lm_head + (size_t)c->code_base * m.d, m.d, ITEM_ROWS, 64, eb, sizeof eb);
+  bool ok = gemm_make_map(&hm[L6], m.lm_head + (size_t)c->code_base * m.d, m.d, ITEM_ROWS, 128, eb, sizeof eb);
   for (int v = 0; v < 2 && ok; ++v) {
     const int bn = v == 0 ? 128 : 256;
     ok = gemm_make_map(&hm[L6 + 1 + 3 * v], m.x, m.d, m.Xrows, bn, eb, sizeof eb) &&

@@ -142,18 +142,14 @@ __device__ __forceinline__ GP gemm_phase(const FwdParams& p, int gi, int BN) {
   return g;
 }
 
-// Weight-tile coordinates of (tile, k-block): k offset and the rows of the two 64-row boxes
-// (SwiGLU tiles pair 64 gate rows with the matching 64 up rows).
-__device__ __forceinline__ void a_coords(const GP& g, int tile, int kbi, int& x, int& y0, int& y1) {
-  const int mt = tile / g.n_tiles;
-  x = kbi * GEMM_BK;
-  if (g.epi == EPI_SWIGLU) {
-    y0 = mt * 64;
-    y1 = g.up_row0 + mt * 64;
-  } else {
-    y0 = mt * GEMM_BM;
-    y1 = mt * GEMM_BM + 64;
-  }
+// Copy of one stage of weight tile mt: 128 rows x 64 k, one box (SwiGLU: 64 gate rows and the
+// matching 64 up rows of a three-dimensional map [gate | up][d_ffn][d]).
+__device__ __forceinline__ void load_weights(const GP& g, const CUtensorMap* map, uint8_t* dst, uint64_t* bar, int mt,
+                                             int kx, uint64_t pol) {
+  if (g.epi == EPI_SWIGLU)
+    tma_load_3d_cg<1>(dst, map, smem_u32(bar), kx, mt * 64, 0, pol);
+  else
+    tma_load_2d(dst, map, bar, kx, mt * GEMM_BM, pol);
 }
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* a) {
@@ -696,7 +692,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
     // ------------------------------------------------------------- weight producer (never waits for the grid)
     if (lane == 0) {
       const uint64_t pol = policy_evict_first();
-      long long n = 0;
+      int s = 0;
+      uint32_t ph = 0;
       bool ok = true;
       for (int gi = 0; gi < NG && ok; ++gi) {
         const GP g = gemm_phase(p, gi, BN);
@@ -705,20 +702,19 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
         it.init(g.w, c);
         int tile, k0, k1;
         while (ok && it.next(g.w, tile, k0, k1)) {
-          int kx, r0, r1;
-          a_coords(g, tile, k0, kx, r0, r1);
-          for (int kbi = k0; kbi < k1; ++kbi, ++n, kx += GEMM_BK) {
-            const int s = (int)(n % C::SA);
-            const uint32_t ph = (uint32_t)((n / C::SA) & 1);
+          const int mt = tile / g.n_tiles;
+          for (int kbi = k0; kbi < k1; ++kbi) {
             if (!mwait(&emptyA[s], ph ^ 1u, p.err)) {
               ok = false;
               break;
             }
-            uint8_t* sa = ringA + s * C::A_BYTES;
             mbar_arrive_expect_tx(&fullA[s], C::A_BYTES);
             lastA[s] = (int)ph;
-            tma_load_2d(sa, mA, &fullA[s], kx, r0, pol);
-            tma_load_2d(sa + 8192, mA, &fullA[s], kx, r1, pol);
+            load_weights(g, mA, ringA + s * C::A_BYTES, &fullA[s], mt, kbi * GEMM_BK, pol);
+            if (++s == C::SA) {
+              s = 0;
+              ph ^= 1u;
+            }
           }
         }
       }
@@ -728,7 +724,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
     // ------------------------------------------------------------- activation producer
     if (lane == 0) {
       const uint64_t pol = policy_evict_last();
-      long long n = 0;
+      int s = 0;
+      uint32_t ph = 0;
       bool ok = true;
       for (int gi = 0; gi < NG && ok; ++gi) {
         const GP g = gemm_phase(p, gi, BN);
@@ -748,9 +745,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
         int tile, k0, k1;
         while (ok && it.next(g.w, tile, k0, k1)) {
           const int nt = tile % g.n_tiles;
-          for (int kbi = k0; kbi < k1; ++kbi, ++n) {
-            const int s = (int)(n % C::SB);
-            const uint32_t ph = (uint32_t)((n / C::SB) & 1);
+          for (int kbi = k0; kbi < k1; ++kbi) {
             if (!mwait(&emptyB[s], ph ^ 1u, p.err)) {
               ok = false;
               break;
@@ -758,6 +753,10 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
             mbar_arrive_expect_tx(&fullB[s], C::B_BYTES);
             lastB[s] = (int)ph;
             tma_load_2d(ringB + s * C::B_BYTES, mB, &fullB[s], kbi * GEMM_BK, nt * BN, pol);
+            if (++s == C::SB) {
+              s = 0;
+              ph ^= 1u;
+            }
           }
         }
         if (p.trace) p.trace[((size_t)2 * (7 * L + 2) + gi) * G + c] = globaltimer_ns();
@@ -768,7 +767,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
     // ------------------------------------------------------------- MMA issuer
     if (lane == 0) {
       constexpr uint32_t idesc = idesc_bf16_f32(GEMM_BM, BN);
-      long long n = 0;
+      int sa = 0, sb = 0;
+      uint32_t pa = 0, pb = 0;
       int si = 0;
       int mma_waits = 0;
       bool ok = true;
@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
         bool any = false;
         while (ok && it.next(g.w, tile, k0, k1)) {
           any = true;
-          const long long len = k1 - k0;
+          const int len = k1 - k0;
           const int acc = si & 1, use = si >> 1;
           ++si;
           if (!mwait(&tempty[acc], (uint32_t)(use & 1) ^ 1u, p.err)) {
@@ -789,9 +789,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
           }
           tc_fence_after();
           const uint32_t dt = tmem_base + (uint32_t)(acc * BN);
-          for (long long j = 0; j < len; ++j, ++n) {
-            const int sa = (int)(n % C::SA), sb = (int)(n % C::SB);
-            const uint32_t pa = (uint32_t)((n / C::SA) & 1), pb = (uint32_t)((n / C::SB) & 1);
+          for (int j = 0; j < len; ++j) {
             if (!mwait(&fullA[sa], pa, p.err) || !mwait(&fullB[sb], pb, p.err)) {
               ok = false;
               break;
@@ -804,6 +802,14 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
               tc_mma_bf16(dt, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc, (j > 0 || kk > 0) ? 1u : 0u);
             tc_commit(&emptyA[sa]);
             tc_commit(&emptyB[sb]);
+            if (++sa == C::SA) {
+              sa = 0;
+              pa ^= 1u;
+            }
+            if (++sb == C::SB) {
+              sb = 0;
+              pb ^= 1u;
+            }
           }
           if (!ok) break;
           tc_commit(&tfull[acc]);

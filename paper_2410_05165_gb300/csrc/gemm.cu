@@ -326,18 +326,19 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-bool make_map(CUtensorMap* m, const void* base, int inner, int rows, int box_rows, char* eb, size_t el) {
+// halves = 1: [rows][inner], box {64, box_rows}; halves = 2: [2][rows][inner], box {64, box_rows, 2}.
+bool make_map(CUtensorMap* m, const void* base, int inner, int rows, int box_rows, int halves, char* eb, size_t el) {
   auto fn = encode_fn();
   if (!fn) {
     snprintf(eb, el, "cuTensorMapEncodeTiled unavailable");
     return false;
   }
-  cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)inner * 2};
-  cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
-  cuuint32_t es[2] = {1, 1};
-  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+  cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)halves};
+  cuuint64_t strides[2] = {(cuuint64_t)inner * 2, (cuuint64_t)inner * 2 * (cuuint64_t)rows};
+  cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, (cuuint32_t)halves};
+  cuuint32_t es[3] = {1, 1, 1};
+  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, halves == 1 ? 2 : 3, const_cast<void*>(base), dims, strides, box,
+                  es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     snprintf(eb, el, "cuTensorMapEncodeTiled failed (%d): inner=%d rows=%d box_rows=%d", (int)r, inner, rows,
@@ -428,7 +429,11 @@ cudaError_t lse_combine_launch(const float2* part, int ld, int m_tiles, int T, f
 }
 
 bool gemm_make_map(CUtensorMap* m, const void* base, int inner, int rows, int box_rows, char* eb, size_t el) {
-  return make_map(m, base, inner, rows, box_rows, eb, el);
+  return make_map(m, base, inner, rows, box_rows, 1, eb, el);
+}
+
+bool gemm_make_map_pairs(CUtensorMap* m, const void* base, int inner, int rows, char* eb, size_t el) {
+  return make_map(m, base, inner, rows, 64, 2, eb, el);
 }
 
 size_t gemm_ws_bytes(int grid) { return (size_t)2 * grid * WS_SLOT_FLOATS * sizeof(float); }
@@ -485,8 +490,8 @@ cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaS
   kp.err = s.err;
   CUtensorMap ma, mb;
   // an operand the tensor-map encoder refuses (typically a base address that is not 16-byte aligned)
-  if (!make_map(&ma, a.W, a.K, a.M, 64, eb, el)) return kGemmMapError;
-  if (!make_map(&mb, a.X, a.K, a.X_rows, BN, eb, el)) return kGemmMapError;
+  if (!make_map(&ma, a.W, a.K, a.M, 64, 1, eb, el)) return kGemmMapError;
+  if (!make_map(&mb, a.X, a.K, a.X_rows, BN, 1, eb, el)) return kGemmMapError;
   return BN == 128 ? launch_bn<128>(a.epi, ma, mb, kp, stream, pdl) : launch_bn<256>(a.epi, ma, mb, kp, stream, pdl);
 }
 

@@ -75,6 +75,10 @@ int gemm_grid_size(int device);
 // 2D bf16 tensor map over a row-major [rows][inner] matrix, box {64, box_rows}, 128B swizzle.
 bool gemm_make_map(CUtensorMap* m, const void* base, int inner, int rows, int box_rows, char* eb, size_t el);
 
+// 3D bf16 tensor map over two stacked matrices [2][rows][inner] (gate rows, then up rows), box
+// {64, 64, 2}: one copy brings 64 gate rows and the matching 64 up rows, in that order.
+bool gemm_make_map_pairs(CUtensorMap* m, const void* base, int inner, int rows, char* eb, size_t el);
+
 // gemm_launch's return value when an operand cannot be described by a tensor map (its base
 // address or row pitch breaks the TMA alignment rules); cudaErrorInvalidValue means a bad shape.
 constexpr cudaError_t kGemmMapError = cudaErrorInvalidDevicePointer;
