@@ -13,26 +13,27 @@ namespace atspeed {
 
 namespace {
 
+constexpr int ATT_OP_BUFS = 3;   // K/V buffers of an item
+
 template <int HD>
 __global__ void __launch_bounds__(128)
     attn_prefix_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv,
                        const AttnArgs a) {
-  using C = AttCfg<HD>;
+  using C = AttCfg<HD, ATT_OP_BUFS>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::SMEM_BODY);
   pdl_launch_dependents();
   pdl_wait();
   if (threadIdx.x == 0) {
-    mbar_init(&bars[0], 1);
-    mbar_init(&bars[1], 1);
+    for (int b = 0; b < ATT_OP_BUFS; ++b) mbar_init(&bars[b], 1);
     fence_mbar_init();
     tma_prefetch_desc(&mk);
     tma_prefetch_desc(&mv);
   }
   __syncthreads();
-  int use[2] = {0, 0};
-  attn_item<HD>(a, &mk, &mv, blockIdx.x, blockIdx.y, blockIdx.z, smem, bars, use, threadIdx.x, 1);
+  uint32_t par = 0;
+  attn_item<HD, ATT_OP_BUFS>(a, &mk, &mv, blockIdx.x, blockIdx.y, blockIdx.z, smem, bars, par, threadIdx.x, 1);
 }
 
 // One CTA of 128 threads per (query tile, head, group of 16 queries): merge the prefix splits with
@@ -59,7 +60,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn_att() {
 
 template <int HD>
 cudaError_t launch_hd(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t st, bool pdl) {
-  using C = AttCfg<HD>;
+  using C = AttCfg<HD, ATT_OP_BUFS>;
   static std::atomic<unsigned long long> attr_done{0};
   {
     const cudaError_t e = smem_attr_once(attr_done, attn_prefix_kernel<HD>, C::SMEM);

@@ -59,34 +59,36 @@ __device__ __forceinline__ int q_chunk(int r, int c) {
   return c ^ (r & ((HD / 8 < 8 ? HD / 8 : 8) - 1));
 }
 
-template <int HD>
+template <int HD, int D>
 struct AttCfg {
-  // SMEM_BODY: bytes from the 1024-aligned base: the K/V double buffer (half pages of ATT_SUB keys);
-  // the Q tile (rows of HD bf16, 16-byte chunks XOR-swizzled by row) is staged in the second
+  // SMEM_BODY: bytes from the 1024-aligned base: the ring of D K/V buffers (half pages of ATT_SUB
+  // keys); the Q tile (rows of HD bf16, 16-byte chunks XOR-swizzled by row) is staged in the last
   // buffer before its first K/V copy (Q lives in registers from then on)
   static constexpr int Q_BYTES = ATT_QTILE * HD * 2;
   static constexpr int KV_BYTES = ATT_SUB * HD * 2;          // one K (or V) half-page tile
   static constexpr int BUF_BYTES = 2 * KV_BYTES;             // K + V
-  static constexpr int SMEM_BODY = 2 * BUF_BYTES;
+  static constexpr int SMEM_BODY = D * BUF_BYTES;
   static_assert(Q_BYTES <= BUF_BYTES, "the Q tile must fit in one K/V buffer");
   static constexpr int SMEM = 1024 + SMEM_BODY + 64;
 };
 
 // One work item (query tile, head, prefix split) with 128 threads (4 warps, 16 queries each).
-// smem: 1024-aligned, AttCfg<HD>::SMEM_BODY bytes; bars: two mbarriers initialised by the caller
-// (count 1) whose completed uses are tracked in use[0], use[1] identically by every thread.
-// Writes the normalised output (a.direct) or the split's unnormalised partials.  Returns false if
-// a bounded wait timed out.
-template <int HD>
+// smem: 1024-aligned, AttCfg<HD, D>::SMEM_BODY bytes; bars: D mbarriers initialised by the caller
+// (count 1); par: bit b is the parity of buffer b's next fill (zero at first), kept identically by
+// every thread from item to item.  Writes the normalised output (a.direct) or the split's
+// unnormalised partials.  Returns false if a bounded wait timed out.
+// D - 1 copies are in flight ahead of the arithmetic: a step of 32 keys takes ~0.5 us of tensor and
+// softmax work, a copy 1.5 - 2 us (more from DRAM), so two buffers left the warps waiting for copies.
+template <int HD, int D>
 __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtensorMap* mv, int tile, int h, int split,
-                          uint8_t* smem, uint64_t* bars, int (&use)[2], int tid, int bar_id,
+                          uint8_t* smem, uint64_t* bars, uint32_t& par, int tid, int bar_id,
                           unsigned long long* tr = nullptr, size_t trs = 0) {
 #define ATT_TR(k) do { if (tr && tid == 0) tr[(size_t)(k) * trs] = globaltimer_ns(); } while (0)
-  using C = AttCfg<HD>;
+  using C = AttCfg<HD, D>;
   constexpr int NDT = HD / 8;    // dim n-tiles of O
   constexpr int NKS = HD / 16;   // k-steps of Q K^T
-  uint8_t* kvbuf = smem;                                             // [2][K | V]
-  __nv_bfloat16* qs = reinterpret_cast<__nv_bfloat16*>(smem + C::BUF_BYTES);   // buffer 1, until chunk 2's copy
+  uint8_t* kvbuf = smem;                                             // [D][K | V]
+  __nv_bfloat16* qs = reinterpret_cast<__nv_bfloat16*>(smem + (D - 1) * C::BUF_BYTES);   // last buffer, until its copy
   const int warp = tid >> 5, lane = tid & 31;
   const int d = a.n_heads * HD;
   const int u = a.qt_user[tile];
@@ -106,11 +108,19 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
     c1 = min(nch, c0 + a.chunks_per_split);
   }
   ATT_TR(0);
-  int page0 = 0, page1 = 0;   // cache pages of the first two pages (thread 0)
-  // copy of half page sc (keys sc * ATT_SUB ...) into buffer buf
-  auto issue = [&](int sc, int buf) {
-    const int pg = sc / (ATT_PAGE / ATT_SUB);
-    const int row0 = (pg == c0 ? page0 : pg == c0 + 1 ? page1 : ptab[pg]) * ATT_PAGE + (sc % (ATT_PAGE / ATT_SUB)) * ATT_SUB;
+  constexpr int SUBS = ATT_PAGE / ATT_SUB;
+  static_assert(SUBS == 2, "copies alternate between a page's halves");
+  const int nst = (c1 - c0) * SUBS;   // steps: half pages
+  // copies are issued in order by thread 0: half page `is` of the item next, page ids read a page ahead
+  int is = 0, page = 0, page_next = 0;
+  auto issue = [&](int buf) {
+    if ((is & 1) == 0) {
+      page = page_next;
+      const int pn = c0 + is / SUBS + 1;
+      if (pn < c1) page_next = ptab[pn];
+    }
+    const int row0 = page * ATT_PAGE + (is & 1) * ATT_SUB;
+    ++is;
     uint8_t* kb = kvbuf + buf * C::BUF_BYTES;
     mbar_arrive_expect_tx(&bars[buf], C::BUF_BYTES);
     const uint64_t pol = policy_evict_last();
@@ -119,12 +129,10 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
       tma_load_2d(kb + C::KV_BYTES + b * (ATT_SUB * BOXW * 2), mv, &bars[buf], h * HD + b * BOXW, row0, pol);
     }
   };
-  constexpr int SUBS = ATT_PAGE / ATT_SUB;
-  // the first K / V half page does not depend on Q: start its copy now
-  if (tid == 0 && c0 < c1) {
-    page0 = ptab[c0];
-    if (c0 + 1 < c1) page1 = ptab[c0 + 1];
-    issue(c0 * SUBS, 0);
+  // the first K / V half pages do not depend on Q: start their copies now
+  if (tid == 0 && nst > 0) {
+    page_next = ptab[c0];
+    for (int b = 0; b < D - 1 && b < nst; ++b) issue(b);
   }
   // Q tile -> shared memory (rows >= nq are zero); all of a thread's loads are issued first
   {
@@ -158,7 +166,6 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
       ldsm_x4(qbase + (uint32_t)((r * HD + q_chunk<HD>(r, kk * 2 + cofs) * 8) * 2), qf[kk][0], qf[kk][1], qf[kk][2],
               qf[kk][3]);
   }
-  named_bar_sync(bar_id, 128);   // every warp holds its Q fragments: buffer 1 may receive K/V now
   const int g = lane >> 2, tq = lane & 3;
   const int row_a = warp * 16 + g, row_b = row_a + 8;
   const int vis_a = row_a < nq ? a.tok_vis[t0 + row_a] : 0;
@@ -171,16 +178,19 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
   float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
   bool ok = true;
 
-  for (int sc = c0 * SUBS; sc < c1 * SUBS; ++sc) {
-    const int buf = (sc - c0 * SUBS) & 1;
-    if (tid == 0 && sc + 1 < c1 * SUBS) issue(sc + 1, buf ^ 1);
-    const bool got = named_bar_and(bar_id, 128, mbar_wait(&bars[buf], (uint32_t)(use[buf] & 1), a.err));
-    if (sc - c0 * SUBS < 2) ATT_TR(2 + 2 * (sc - c0 * SUBS));
-    ++use[buf];
+  int buf = 0;
+  for (int st = 0; st < nst; ++st) {
+    // (the vote is also the barrier after which every warp has read the previous step's buffer -- at
+    // the first step the Q tile --, which the next copy fills)
+    const bool got = named_bar_and(bar_id, 128, mbar_wait(&bars[buf], (par >> buf) & 1u, a.err));
+    if (st < 2) ATT_TR(2 + 2 * st);
     if (!got) {
       ok = false;
       break;
     }
+    par ^= 1u << buf;
+    if (tid == 0 && is < nst) issue(buf == 0 ? D - 1 : buf - 1);
+    const int sc = c0 * SUBS + st;
     const uint32_t kbase = smem_u32(kvbuf + buf * C::BUF_BYTES);
     const uint32_t vbase = kbase + C::KV_BYTES;
     {
@@ -260,17 +270,20 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
         }
       }
     }
-    named_bar_sync(bar_id, 128);  // buffer `buf` may be refilled next iteration
-    if (sc - c0 * SUBS < 2) ATT_TR(3 + 2 * (sc - c0 * SUBS));
+    if (++buf == D) buf = 0;
+    if (st < 2) ATT_TR(3 + 2 * st);
   }
   if (!ok) {
-    // the copy for the next chunk may still be in flight: wait for it (bounded) before returning
+    // copies ahead of the failed step may still be in flight: wait for them (bounded; a buffer that
+    // has none runs into its limit) before returning
     if (tid == 0) {
-      for (int b = 0; b < 2; ++b) mbar_wait(&bars[b], (uint32_t)(use[b] & 1), nullptr);
+      for (int b = 0; b < D; ++b) mbar_wait(&bars[b], (par >> b) & 1u, nullptr, kDrainNs);
     }
     named_bar_sync(bar_id, 128);
     return false;
   }
+  // the next item's copies and Q tile overwrite the buffers: every warp is done with the last ones
+  named_bar_sync(bar_id, 128);
   l_a += __shfl_xor_sync(0xffffffffu, l_a, 1);
   l_a += __shfl_xor_sync(0xffffffffu, l_a, 2);
   l_b += __shfl_xor_sync(0xffffffffu, l_b, 1);

@@ -59,7 +59,9 @@ struct FCfg {
   static constexpr int A_BYTES = GEMM_BM * 128;
   static constexpr int B_BYTES = BN * 128;
   static constexpr int STAGING = 2 * 32 * GEMM_BM * 4;   // one [32][128] fp32 chunk per warpgroup
-  static constexpr int MISC = 8192;
+  static constexpr int TABLES = 4096;                    // part slots, token tables, norm scales
+  static constexpr int MISC = 1536;                      // barriers, flags, epilogue arguments
+  static constexpr int AD = BN == 128 ? 3 : 4;           // K/V buffers of a warpgroup's attention item
   static constexpr int TMEM_COLS = 2 * BN;
 };
 
@@ -69,15 +71,15 @@ struct FLayout {
   static constexpr int A_OFF = 0;
   static constexpr int B_OFF = C::SA * C::A_BYTES;
   static constexpr int STG_OFF = B_OFF + C::SB * C::B_BYTES;
-  // the attention work areas (one per warpgroup) overlap the activation ring and the staging buffers
-  // (both idle then)
+  static constexpr int TAB_OFF = STG_OFF + C::STAGING;
+  // the attention work areas (one per warpgroup) overlap the activation ring, the staging buffers and
+  // the GEMM phases' tables (all idle then)
   static constexpr int ATT_OFF = B_OFF;
-  static constexpr int ATT_BODY = ((AttCfg<HD>::SMEM_BODY + 1023) / 1024) * 1024;
-  static constexpr int ATT_NEED = 2 * ATT_BODY;
-  static constexpr int AFTER_STG = STG_OFF + C::STAGING;
-  static constexpr int EXTRA = (ATT_OFF + ATT_NEED > AFTER_STG) ? ((ATT_OFF + ATT_NEED - AFTER_STG + 1023) / 1024) * 1024 : 0;
-  static constexpr int MISC_OFF = AFTER_STG + EXTRA;
+  static constexpr int ATT_BODY = ((AttCfg<HD, C::AD>::SMEM_BODY + 1023) / 1024) * 1024;
+  static constexpr int ATT_END = ATT_OFF + 2 * ATT_BODY;
+  static constexpr int MISC_OFF = TAB_OFF + C::TABLES > ATT_END ? TAB_OFF + C::TABLES : ATT_END;
   static constexpr int TOTAL = 1024 + MISC_OFF + C::MISC;
+  static_assert(TOTAL <= 232448, "shared memory of a CTA");
   static_assert(C::SB * C::B_BYTES >= 8192 * 4, "a final-norm row (d <= 8192 floats) must fit in the activation ring");
 };
 
@@ -366,9 +368,9 @@ __device__ __forceinline__ void norm_phase(const FwdParams& p, bool final, const
 // Tree attention of layer l, one warpgroup (128 threads, `wt`): its work items (query tile, head,
 // prefix split) are item c + (2k + wg) G; each is followed by the warpgroup's share of the merge of
 // the splits of (tile, head) once all of them are published.
-template <int HD>
+template <int HD, int AD>
 __device__ __forceinline__ bool attn_phase(const FwdParams& p, int l, uint8_t* att_smem, uint64_t* att_bars,
-                                           int (&use_att)[2], int* flag, int wt, int wg, int wbar) {
+                                           uint32_t& att_par, int* flag, int wt, int wg, int wbar) {
   const int c = blockIdx.x, G = p.G, L = p.L;
   AttnArgs a = p.att_args;
   a.k_cache = p.kc + p.layer_elems * l;
@@ -383,7 +385,7 @@ __device__ __forceinline__ bool attn_phase(const FwdParams& p, int l, uint8_t* a
     const int h = rem / S, split = rem % S;
     const bool tr_on = p.trace && wg == 0 && nit == 0;
     unsigned long long* tr = tr_on ? p.trace + ((size_t)8 * NP + ph) * G + c : nullptr;
-    if (!attn_item<HD>(a, mk, mv, tile, h, split, att_smem, att_bars, use_att, wt, wbar, tr, (size_t)NP * G))
+    if (!attn_item<HD, AD>(a, mk, mv, tile, h, split, att_smem, att_bars, att_par, wt, wbar, tr, (size_t)NP * G))
       return false;
     if (tr_on && wt == 0) p.trace[((size_t)4 * NP + ph) * G + c] = globaltimer_ns();
     if (a.direct) continue;
@@ -630,8 +632,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
   uint64_t* tfull = emptyB + C::SB;
   uint64_t* tempty = tfull + 2;
   uint64_t* mma_done = tempty + 2;
-  uint64_t* att_bars = mma_done + 1;                              // 2 per warpgroup
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(att_bars + 4);
+  uint64_t* att_bars = mma_done + 1;                              // AD per warpgroup
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(att_bars + 2 * C::AD);
   int* flag = reinterpret_cast<int*>(tmem_slot + 1);
   int* flagw = flag + 1;                                          // 2: one per warpgroup
   int* failed = flagw + 2;
@@ -639,15 +641,15 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
   int* lastA = go + 1;                                            // [SA] parity of last fill, -1 none
   int* lastB = lastA + C::SA;                                     // [SB]
   float* red = reinterpret_cast<float*>(lastB + C::SB);           // 8
-  int* part_slot = reinterpret_cast<int*>(red + 8);               // 256
+  GemmArgs* s_ea = reinterpret_cast<GemmArgs*>((reinterpret_cast<uintptr_t>(red + 8) + 15) &
+                                                ~uintptr_t(15));   // epilogue arguments
+  static_assert(8 * (2 * C::SA + 2 * C::SB + 5 + 2 * C::AD) + 4 * (6 + C::SA + C::SB + 8) + 16 + (int)sizeof(GemmArgs) <=
+                    C::MISC,
+                "shared-memory misc area too small");
+  int* part_slot = reinterpret_cast<int*>(smem + LY::TAB_OFF);    // 256
   int* tpos = part_slot + 256;                                    // [BN] QKV token tables
   int* tkvr = tpos + 256;
   float* trs = reinterpret_cast<float*>(tkvr + 256);              // [BN] norm scales (QKV, gate/up)
-  GemmArgs* s_ea = reinterpret_cast<GemmArgs*>((reinterpret_cast<uintptr_t>(trs + 256) + 15) &
-                                                ~uintptr_t(15));   // epilogue arguments
-  static_assert(8 * (2 * C::SA + 2 * C::SB + 9) + 4 * (6 + C::SA + C::SB + 8 + 256 + 768) + 16 + (int)sizeof(GemmArgs) <=
-                    C::MISC,
-                "shared-memory misc area too small");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = blockIdx.x, G = p.G, L = p.L;
@@ -669,7 +671,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
       mbar_init(&tfull[i], 1);
       mbar_init(&tempty[i], 8);   // one arrival per compute warp
     }
-    for (int i = 0; i < 4; ++i) mbar_init(&att_bars[i], 1);
+    for (int i = 0; i < 2 * C::AD; ++i) mbar_init(&att_bars[i], 1);
     mbar_init(mma_done, 1);
     *go = 0;
     *failed = 0;
@@ -833,7 +835,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
     const int ctid = threadIdx.x - COMPUTE_WARP0 * 32;
     const int wg = ctid >> 7, wt = ctid & 127;
     int si = 0;
-    int use_att[2] = {0, 0};
+    uint32_t att_par = 0;
     bool ok = true;
     int nb = 0;   // grid barriers passed
     for (int ph = 0; ph < NP && ok; ++ph) {
@@ -883,8 +885,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
         norm_phase<BN>(p, kind == 4, kind == 0 ? p.attn_norm[0] : p.final_norm, red, rowbuf, ctid, ph);
       } else if (kind == 2) {
         // both warpgroups leave together: a failed bounded wait in either ends the program
-        const bool aok = attn_phase<HD>(p, l, att_smem + wg * LY::ATT_BODY, att_bars + 2 * wg,
-                                        use_att, flagw + wg, wt, wg, 2 + wg);
+        const bool aok = attn_phase<HD, C::AD>(p, l, att_smem + wg * LY::ATT_BODY, att_bars + C::AD * wg, att_par,
+                                               flagw + wg, wt, wg, 2 + wg);
         if (!named_bar_and(1, CT, aok)) {
           ok = false;
           break;
