@@ -22,35 +22,45 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t& r0, uint32_t&
                : "r"(addr));
 }
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
+  asm(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 __device__ __forceinline__ void mma_f16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
+  asm(
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&v);
+// 2^x with the hardware's approximation (results below the smallest normal number flush to zero: such a
+// weight, against the row maximum's 1, changes no sum)
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
-// Byte offset of (row, 16-byte chunk) inside a K or V tile of ATT_SUB rows as written by TMA.
-// HD >= 64: boxes of 64 columns (128 B rows), 128-byte swizzle: chunk ^= row & 7.
-// HD == 32: one box of 64-byte rows, no swizzle.
+// K and V tiles of ATT_SUB rows as written by TMA.  HD >= 64: boxes of 64 columns (128-byte rows),
+// 128-byte swizzle: 16-byte chunk c of row r sits at chunk c ^ (r & 7).  HD == 32: one box of 64-byte
+// rows, no swizzle.
+// frag_base: address of (row, chunk b) with b in {0, 1}; frag_addr: from it, that of (row + 16 rows16,
+// chunk + b) with an even `chunk` (only bits 4-6 of the swizzled address depend on it: one xor).
 template <int HD>
-__device__ __forceinline__ uint32_t kv_off(int row, int chunk16) {
-  if constexpr (HD >= 64) {
-    const int box = chunk16 >> 3, c = chunk16 & 7;
-    return (uint32_t)(box * (ATT_SUB * 128) + row * 128 + ((c ^ (row & 7)) << 4));
-  } else {
-    return (uint32_t)(row * (HD * 2) + (chunk16 << 4));
-  }
+__device__ __forceinline__ uint32_t frag_base(uint32_t tile, int row, int b) {
+  if constexpr (HD >= 64)
+    return tile + (uint32_t)(row * 128 + ((b ^ (row & 7)) << 4));
+  else
+    return tile + (uint32_t)(row * (HD * 2) + (b << 4));
+}
+template <int HD>
+__device__ __forceinline__ uint32_t frag_addr(uint32_t base, int chunk, int rows16) {
+  if constexpr (HD >= 64)
+    return (base ^ (uint32_t)((chunk & 7) << 4)) + (uint32_t)((chunk >> 3) * (ATT_SUB * 128) + rows16 * 16 * 128);
+  else
+    return base + (uint32_t)((chunk << 4) + rows16 * 16 * (HD * 2));
 }
 
 // Physical 16-byte chunk of logical chunk c of Q row r (conflict-free ldmatrix without padding).
@@ -171,6 +181,15 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
   const int vis_a = row_a < nq ? a.tok_vis[t0 + row_a] : 0;
   const int vis_b = row_b < nq ? a.tok_vis[t0 + row_b] : 0;
   const float scale = kLog2e / sqrtf((float)HD);
+  // keys below vis_full are visible to every query of the warp (rows past the tile's last query are
+  // not stored and do not count)
+  int vis_full = min(row_a < nq ? vis_a : 0x7fffffff, row_b < nq ? vis_b : 0x7fffffff);
+#pragma unroll
+  for (int i = 16; i > 0; i >>= 1) vis_full = min(vis_full, __shfl_xor_sync(0xffffffffu, vis_full, i));
+  // ldmatrix rows of this lane in buffer 0: K (keys (lane & 7) + 8 (lane / 16), 8-dimension halves by lane
+  // bit 3), V (keys (lane & 7) + 8 (lane bit 3), halves by lane / 16)
+  const uint32_t kf0 = frag_base<HD>(smem_u32(kvbuf), (lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1);
+  const uint32_t vf0 = frag_base<HD>(smem_u32(kvbuf) + C::KV_BYTES, (lane & 7) + (((lane >> 3) & 1) << 3), lane >> 4);
 
   float o[NDT][4];
 #pragma unroll
@@ -191,36 +210,67 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
     par ^= 1u << buf;
     if (tid == 0 && is < nst) issue(buf == 0 ? D - 1 : buf - 1);
     const int sc = c0 * SUBS + st;
-    const uint32_t kbase = smem_u32(kvbuf + buf * C::BUF_BYTES);
-    const uint32_t vbase = kbase + C::KV_BYTES;
+    const uint32_t koff = kf0 + (uint32_t)(buf * C::BUF_BYTES), voff = vf0 + (uint32_t)(buf * C::BUF_BYTES);
     {
-      constexpr int hk = 0;   // the buffer holds the half page's ATT_SUB = 32 keys
       float s[4][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) s[j][0] = s[j][1] = s[j][2] = s[j][3] = 0.f;
+      // Q K^T and P V in batches of four fragment loads, each batch's loads issued before the previous
+      // batch's MMAs; the four score accumulators (sixteen output ones) are independent chains
+      uint32_t f[2][4][4];
+      auto load_k = [&](int b) {   // fragments of k-steps 2 b, 2 b + 1: keys 0 .. 15 and 16 .. 31
 #pragma unroll
-      for (int jj = 0; jj < 2; ++jj) {
+        for (int i = 0; i < 4; ++i) {
+          const int kk = 2 * b + (i >> 1), jj = i & 1;
+          uint32_t(&r)[4] = f[b & 1][i];
+          ldsm_x4(frag_addr<HD>(koff, kk * 2, jj), r[0], r[1], r[2], r[3]);
+        }
+      };
+      auto load_v = [&](int b) {   // fragments 4 b .. 4 b + 3 of (16 keys, 16 dimensions)
 #pragma unroll
-        for (int kk = 0; kk < NKS; ++kk) {
-          // matrices: (keys 16jj+0..7, dims lo), (keys 0..7, dims hi), (keys 8..15, lo), (keys 8..15, hi)
-          const int key = hk * 32 + jj * 16 + (lane & 7) + ((lane >> 4) << 3);
-          const int ch = kk * 2 + ((lane >> 3) & 1);
-          uint32_t b0, b1, b2, b3;
-          ldsm_x4(kbase + kv_off<HD>(key, ch), b0, b1, b2, b3);
-          mma_bf16_16816(s[2 * jj], qf[kk], b0, b1);
-          mma_bf16_16816(s[2 * jj + 1], qf[kk], b2, b3);
+        for (int i = 0; i < 4; ++i) {
+          const int n = 4 * b + i, kk = n / (NDT / 2), dd = n % (NDT / 2);
+          uint32_t(&r)[4] = f[b & 1][i];
+          ldsm_x4_t(frag_addr<HD>(voff, dd * 2, kk), r[0], r[1], r[2], r[3]);
+        }
+      };
+      constexpr int NKB = NKS / 2, NVB = NDT / 4;   // batches
+      load_k(0);
+#pragma unroll
+      for (int b = 0; b < NKB; ++b) {
+        if (b + 1 < NKB) load_k(b + 1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int kk = 2 * b + (i >> 1), jj = i & 1;
+          const uint32_t(&r)[4] = f[b & 1][i];
+          mma_bf16_16816(s[2 * jj], qf[kk], r[0], r[1]);
+          mma_bf16_16816(s[2 * jj + 1], qf[kk], r[2], r[3]);
         }
       }
+      load_v(0);   // (in flight during the softmax)
       // scale, mask, online softmax (base 2)
       const int kbase_idx = sc * ATT_SUB;
+      if (kbase_idx + ATT_SUB > vis_full) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int k0 = kbase_idx + j * 8 + tq * 2;
+          s[j][0] = (k0 < vis_a) ? s[j][0] * scale : -INFINITY;
+          s[j][1] = (k0 + 1 < vis_a) ? s[j][1] * scale : -INFINITY;
+          s[j][2] = (k0 < vis_b) ? s[j][2] * scale : -INFINITY;
+          s[j][3] = (k0 + 1 < vis_b) ? s[j][3] * scale : -INFINITY;
+        }
+      } else {   // every key is visible to every query of the warp
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          s[j][0] *= scale;
+          s[j][1] *= scale;
+          s[j][2] *= scale;
+          s[j][3] *= scale;
+        }
+      }
       float mx_a = m_a, mx_b = m_b;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int k0 = kbase_idx + j * 8 + tq * 2;
-        s[j][0] = (k0 < vis_a) ? s[j][0] * scale : -INFINITY;
-        s[j][1] = (k0 + 1 < vis_a) ? s[j][1] * scale : -INFINITY;
-        s[j][2] = (k0 < vis_b) ? s[j][2] * scale : -INFINITY;
-        s[j][3] = (k0 + 1 < vis_b) ? s[j][3] * scale : -INFINITY;
         mx_a = fmaxf(mx_a, fmaxf(s[j][0], s[j][1]));
         mx_b = fmaxf(mx_b, fmaxf(s[j][2], s[j][3]));
       }
@@ -230,7 +280,7 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
       mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 2));
       const float ua = (mx_a == -INFINITY) ? 0.f : mx_a;
       const float ub = (mx_b == -INFINITY) ? 0.f : mx_b;
-      const float alpha_a = exp2f(m_a - ua), alpha_b = exp2f(m_b - ub);
+      const float alpha_a = ex2(m_a - ua), alpha_b = ex2(m_b - ub);
       m_a = mx_a;
       m_b = mx_b;
       l_a *= alpha_a;
@@ -245,8 +295,8 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
       uint32_t ph[2][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float p0 = exp2f(s[j][0] - ua), p1 = exp2f(s[j][1] - ua);
-        const float p2 = exp2f(s[j][2] - ub), p3 = exp2f(s[j][3] - ub);
+        const float p0 = ex2(s[j][0] - ua), p1 = ex2(s[j][1] - ua);
+        const float p2 = ex2(s[j][2] - ub), p3 = ex2(s[j][3] - ub);
         l_a += p0 + p1;
         l_b += p2 + p3;
         const int kk = j >> 1, r = (j & 1) * 2;
@@ -257,16 +307,14 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
       // O += P V with P in fp16 (11 significant bits; the row sum l uses the fp32 values) and V fp16
       // (exactly the bf16-rounded values)
 #pragma unroll
-      for (int kk = 0; kk < 2; ++kk) {
+      for (int b = 0; b < NVB; ++b) {
+        if (b + 1 < NVB) load_v(b + 1);
 #pragma unroll
-        for (int dd = 0; dd < NDT / 2; ++dd) {
-          // trans matrices: (keys 16kk+0..7, dims 16dd+0..7), (keys +8..15, same), (keys 0..7, dims +8..15), (8..15, +8..15)
-          const int key = hk * 32 + kk * 16 + (lane & 7) + (((lane >> 3) & 1) << 3);
-          const int ch = dd * 2 + (lane >> 4);
-          uint32_t b0, b1, b2, b3;
-          ldsm_x4_t(vbase + kv_off<HD>(key, ch), b0, b1, b2, b3);
-          mma_f16_16816(o[2 * dd], ph[kk], b0, b1);
-          mma_f16_16816(o[2 * dd + 1], ph[kk], b2, b3);
+        for (int i = 0; i < 4; ++i) {
+          const int n = 4 * b + i, kk = n / (NDT / 2), dd = n % (NDT / 2);
+          const uint32_t(&r)[4] = f[b & 1][i];
+          mma_f16_16816(o[2 * dd], ph[kk], r[0], r[1]);
+          mma_f16_16816(o[2 * dd + 1], ph[kk], r[2], r[3]);
         }
       }
     }
