@@ -423,7 +423,7 @@ __device__ __forceinline__ bool attn_phase(const FwdParams& p, int l, uint8_t* a
 //  * shared sums (phases with whole tiles per CTA, whose split tiles come first and finish early;
 //    the O / down projections, whose residual update ends the phase; the LM head, whose tiles have
 //    many short parts): every part publishes, then each part sums a share of its tile's chunks
-//    (chunk ch by part ch mod parts).
+//    (sk_share).
 // Parts are always summed in k order starting from zero, whichever CTA sums them.  The QKV and
 // gate/up epilogues first multiply by each token's norm scale (trs, loaded per token tile).
 template <int BN>
@@ -499,9 +499,11 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
       const bool tr_on = p.trace && ctid == 0 && j == 0;
       if (tr_on) p.trace[((size_t)6 * NP + ph) * G + c] = globaltimer_ns();
       const int nch = min(BN / 32, (g.rows - n_tile * BN + 31) / 32);
+      int ch_lo, ch_hi;   // this CTA's chunks
+      sk_share(g.w, t, c_first, parts, c - c_first, nch, ch_lo, ch_hi);
       if (g.dh_out) {
         // residual updates: both warpgroups on each chunk of this part, 16 tokens each
-        for (int ch = c - c_first; ch < nch; ch += parts) {
+        for (int ch = ch_lo; ch < ch_hi; ++ch) {
           if (ch * 32 + 16 * wg >= g.rows - n_tile * BN) continue;   // (warpgroup-uniform)
           ws_reduce_resnorm_half<RED_PB>(ea, p.ws, part_slot, parts, ch, wg, m_tile, n_tile * BN + ch * 32, wt, staging,
                                          wbar);
@@ -512,7 +514,7 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
         continue;
       }
       int k = 0;
-      for (int ch = c - c_first; ch < nch; ch += parts, ++k) {
+      for (int ch = ch_lo; ch < ch_hi; ++ch, ++k) {
         if ((k & 1) != wg) continue;
         ws_reduce_chunk<1>(p.ws, part_slot, parts, ch, m, staging);
         named_bar_sync(wbar, 128);
