@@ -457,7 +457,7 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
   SegIter it;
   it.init(g.w, c);
   int tile, k0, k1;
-  auto fill_part_slots = [&](long long tu0, int c_first, int parts) {
+  auto fill_part_slots = [&](int tu0, int c_first, int parts) {
     for (int pi = ctid; pi < parts; pi += CT) {
       const int cc = c_first + pi;
       part_slot[pi] = cc * 2 + (sk_start(g.w, cc) >= tu0 ? 0 : 1);
@@ -487,7 +487,7 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
     if (p.trace && ctid == 0) p.trace[((size_t)5 * NP + ph) * G + c] = globaltimer_ns();
     for (int j = 0; j < nsk; ++j) {
       const int t = sk_tile[j];
-      const long long tu0 = (long long)t * kb;
+      const int tu0 = t * kb;
       const int c_first = sk_owner(g.w, tu0);
       const int parts = sk_owner(g.w, tu0 + kb - 1) - c_first + 1;
       const int m_tile = t / g.n_tiles, n_tile = t % g.n_tiles;
@@ -531,10 +531,10 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
     const int m_tile = tile / g.n_tiles, n_tile = tile % g.n_tiles;
     const bool whole = (k0 == 0 && k1 == kb);
     tables(n_tile);
-    long long tu0 = 0;
+    int tu0 = 0;
     int c_first = 0, parts = 1;
     if (!whole) {
-      tu0 = (long long)tile * kb;
+      tu0 = tile * kb;
       c_first = sk_owner(g.w, tu0);
       parts = sk_owner(g.w, tu0 + kb - 1) - c_first + 1;
       fill_part_slots(tu0, c_first, parts);
@@ -733,7 +733,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
       bool ok = true;
       for (int gi = 0; gi < NG && ok; ++gi) {
         const GP g = gemm_phase(p, gi, BN);
-        const long long nu = cta_units(g.w, c);
+        const int nu = cta_units(g.w, c);
         // the compute warps pass the grid barrier that publishes this phase's input and count it in
         // `go` (one grid poller per CTA)
         if (!cta_count_wait(go, gi + 1, p.err)) {

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(192, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = blockIdx.x;
-  const long long nu = cta_units(p.w, c);   // this CTA's units (stream-K units, then whole tiles)
+  const int nu = cta_units(p.w, c);   // this CTA's units (stream-K units, then whole tiles)
   const int kb = p.kb;
 
   if (threadIdx.x == 0) {
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(192, 1)
       tma_prefetch_desc(&tmB);
       const uint64_t pol_w = policy_evict_first();   // weights: streamed once
       const uint64_t pol_x = policy_evict_last();    // activations: re-read by every CTA
-      const long long total = nu;
+      const int total = nu;
       const int npre = (int)(total < C::STAGES ? total : C::STAGES);
       // units in order, walked segment by segment (no per-unit divisions)
       SegIter it;
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(192, 1)
         tma_load_2d(smem + i * C::STAGE_BYTES + C::A_BYTES, &tmB, &full[i], pre_xk[i], pre_brow[i], pol_x);
       int stage = npre % C::STAGES;
       uint32_t phase = (npre == C::STAGES) ? 1u : 0u;
-      for (long long i = npre; i < total; ++i) {
+      for (int i = npre; i < total; ++i) {
         if (!mbar_wait(&empty[stage], phase ^ 1u, p.err)) {
           *failed = 1;
           break;
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(192, 1)
       it.init(p.w, c);
       int tile, k0, k1;
       for (; ok && it.next(p.w, tile, k0, k1); ++si) {
-        const long long len = k1 - k0;
+        const int len = k1 - k0;
         const int acc = si & 1, use = si >> 1;
         if (!mbar_wait(&tempty[acc], (uint32_t)(use & 1) ^ 1u, p.err)) {
           ok = false;
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(192, 1)
         }
         tc_fence_after();
         const uint32_t dt = tmem_base + (uint32_t)(acc * BN);
-        for (long long j = 0; j < len; ++j) {
+        for (int j = 0; j < len; ++j) {
           if (!mbar_wait(&full[stage], phase, p.err)) {
             ok = false;
             break;
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(192, 1)
         if (lane == 0) mbar_arrive(&tempty[acc]);
         __threadfence();
         named_bar_sync(1, 128);
-        const long long tu0 = (long long)tile * kb;
+        const int tu0 = tile * kb;
         const int c_first = sk_owner(p.w, tu0);
         const int c_last = sk_owner(p.w, tu0 + kb - 1);
         const int parts = c_last - c_first + 1;

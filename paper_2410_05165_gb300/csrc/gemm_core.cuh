@@ -21,7 +21,7 @@ constexpr int GEMM_WS_SLOT_FLOATS = 256 * 128;
 // With tiles < G (q = 0) this is plain stream-K over all tiles.
 struct WorkSplit {
   int tiles, kb, q, r;
-  long long Usk;   // stream-K units: r * kb
+  int Usk;         // stream-K units: r * kb (G * Usk fits 32 bits: r < G <= SMs, kb <= 256)
   int Gsk;         // CTAs that get stream-K units: min(G, Usk)
   int G;           // CTAs that take work (any others of the grid idle in this GEMM)
 };
@@ -32,8 +32,8 @@ __host__ __device__ inline WorkSplit work_split(int tiles, int kb, int G) {
   w.kb = kb;
   w.q = tiles / G;
   w.r = tiles - w.q * G;
-  w.Usk = (long long)w.r * kb;
-  w.Gsk = (int)(w.Usk < (long long)G ? w.Usk : (long long)G);
+  w.Usk = w.r * kb;
+  w.Gsk = w.Usk < G ? w.Usk : G;
   w.G = G;
   return w;
 }
@@ -49,18 +49,21 @@ __host__ __device__ inline int gemm_work_ctas(long long tiles, int kb, int grid)
   const long long U = tiles * kb;
   return (int)(U < (long long)grid ? U : (long long)grid);
 }
+// (unsigned 32-bit divisions: the 64-bit ones took a visible part of a small model's phases)
+__device__ __forceinline__ int sk_start(const WorkSplit& w, int c) {
+  return (int)((unsigned)c * (unsigned)w.Usk / (unsigned)w.Gsk);
+}
 // stream-K unit range [a, b) of CTA c
-__device__ __forceinline__ void sk_range(const WorkSplit& w, int c, long long& a, long long& b) {
+__device__ __forceinline__ void sk_range(const WorkSplit& w, int c, int& a, int& b) {
   if (c >= w.Gsk) {
     a = b = 0;
     return;
   }
-  a = (long long)c * w.Usk / w.Gsk;
-  b = (long long)(c + 1) * w.Usk / w.Gsk;
+  a = sk_start(w, c);
+  b = sk_start(w, c + 1);
 }
-__device__ __forceinline__ long long sk_start(const WorkSplit& w, long long c) { return c * w.Usk / w.Gsk; }
-__device__ __forceinline__ int sk_owner(const WorkSplit& w, long long u) {
-  return (int)(((u + 1) * (long long)w.Gsk - 1) / w.Usk);
+__device__ __forceinline__ int sk_owner(const WorkSplit& w, int u) {
+  return (int)(((unsigned)(u + 1) * (unsigned)w.Gsk - 1u) / (unsigned)w.Usk);
 }
 // Shared sums of a split tile: the nch chunks of 32 tokens are dealt out in contiguous ranges over the
 // tile's `parts` CTAs (c_first ..), a CTA that also sums a neighbouring tile getting half the share of
@@ -69,8 +72,8 @@ __device__ __forceinline__ int sk_owner(const WorkSplit& w, long long u) {
 // [lo, hi): the chunks of part `pi`.
 __device__ __forceinline__ void sk_share(const WorkSplit& w, int tile, int c_first, int parts, int pi, int nch, int& lo,
                                          int& hi) {
-  const bool first_shared = sk_start(w, c_first) < (long long)tile * w.kb;
-  const bool last_shared = sk_start(w, c_first + parts) > (long long)(tile + 1) * w.kb;
+  const bool first_shared = sk_start(w, c_first) < tile * w.kb;
+  const bool last_shared = sk_start(w, c_first + parts) > (tile + 1) * w.kb;
   if (parts == 1) {
     lo = 0;
     hi = nch;
@@ -83,31 +86,16 @@ __device__ __forceinline__ void sk_share(const WorkSplit& w, int tile, int c_fir
   lo = (2 * nch * c0 + W) / (2 * W);   // rounded
   hi = (2 * nch * c1 + W) / (2 * W);
 }
-// number of units of CTA c, and its i-th unit as (tile, k-block)
-__device__ __forceinline__ long long cta_units(const WorkSplit& w, int c) {
+// number of units of CTA c
+__device__ __forceinline__ int cta_units(const WorkSplit& w, int c) {
   if (c >= w.G) return 0;
-  long long a, b;
+  int a, b;
   sk_range(w, c, a, b);
-  return (b - a) + (long long)w.q * w.kb;
-}
-__device__ __forceinline__ void cta_unit(const WorkSplit& w, int c, long long i, int& tile, int& kbi) {
-  long long a, b;
-  sk_range(w, c, a, b);
-  if (i < b - a) {
-    const long long u = a + i;
-    tile = (int)(u / w.kb);
-    kbi = (int)(u - (long long)tile * w.kb);
-  } else {
-    const long long j = i - (b - a);
-    const int t = (int)(j / w.kb);
-    tile = w.r + t * w.G + c;
-    kbi = (int)(j - (long long)t * w.kb);
-  }
+  return (b - a) + w.q * w.kb;
 }
 // the segments (one tile's contiguous k-blocks [k0, k1)) of CTA c in order
 struct SegIter {
-  long long u, u1;
-  int dp, dp1;
+  int u, u1, dp, dp1;
   __device__ __forceinline__ void init(const WorkSplit& w, int c) {
     if (c >= w.G) {
       u = u1 = 0;
@@ -120,10 +108,10 @@ struct SegIter {
   }
   __device__ __forceinline__ bool next(const WorkSplit& w, int& tile, int& k0, int& k1) {
     if (u < u1) {
-      tile = (int)(u / w.kb);
-      k0 = (int)(u - (long long)tile * w.kb);
-      const long long len = (w.kb - k0) < (u1 - u) ? (w.kb - k0) : (u1 - u);
-      k1 = k0 + (int)len;
+      tile = (int)((unsigned)u / (unsigned)w.kb);
+      k0 = u - tile * w.kb;
+      const int len = (w.kb - k0) < (u1 - u) ? (w.kb - k0) : (u1 - u);
+      k1 = k0 + len;
       u += len;
       return true;
     }
