@@ -251,13 +251,13 @@ __device__ bool mwait(uint64_t* bar, uint32_t parity, unsigned* err) {
   }
 }
 
-// trs: the n-tile's norm scales (QKV / gate-up); bar: the warpgroup's named barrier (EPI_RESNORM)
+// trs: the n-tile's norm scales (QKV / gate-up).  (The residual updates of the O / down projections have
+// loops of their own.)
 template <int BN>
 __device__ __noinline__ void epi_dispatch(int epi, const GemmArgs* a, float* st, int mt, int nt, int ch, int t,
-                                          const int* tpos, const int* tkvr, const float* trs, int bar) {
+                                          const int* tpos, const int* tkvr, const float* trs) {
   switch (epi) {
     case EPI_F32: epi_chunk<BN, EPI_F32>(*a, st, mt, nt, ch, t, tpos, tkvr); break;
-    case EPI_RESNORM: epi_resnorm(*a, st, mt, nt * BN + ch * 32, t, bar); break;
     case EPI_SWIGLU: epi_chunk<BN, EPI_SWIGLU>(*a, st, mt, nt, ch, t, tpos, tkvr, trs); break;
     default: epi_chunk<BN, EPI_QKV>(*a, st, mt, nt, ch, t, tpos, tkvr, trs); break;
   }
@@ -519,7 +519,7 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
         ws_reduce_chunk<1>(p.ws, part_slot, parts, ch, m, staging);
         named_bar_sync(wbar, 128);
         if (tr_on && k == 0) p.trace[((size_t)8 * NP + ph) * G + c] = globaltimer_ns();
-        epi_dispatch<BN>(g.epi, s_ea, staging, m_tile, n_tile, ch, wt, tpos, tkvr, trs_e, wbar);
+        epi_dispatch<BN>(g.epi, s_ea, staging, m_tile, n_tile, ch, wt, tpos, tkvr, trs_e);
         named_bar_sync(wbar, 128);
         if (tr_on && k == 0) p.trace[((size_t)9 * NP + ph) * G + c] = globaltimer_ns();
       }
@@ -546,6 +546,13 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
     if (p.trace && ctid == 0) p.trace[((size_t)4 * NP + ph) * G + c] = globaltimer_ns();
     const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
     const int nch = min(BN / 32, (g.rows - n_tile * BN + 31) / 32);
+    if (whole && g.dh_out) {
+      // residual updates: both warpgroups on each chunk, 16 tokens each
+      whole_resnorm_half(ea, tb, nch, wg, m_tile, n_tile * BN, wt, m, staging, wbar);
+      tc_fence_before();
+      if (lane == 0) mbar_arrive(&tempty[acc]);
+      continue;
+    }
     if (whole) {
       for (int ch = wg; ch < nch; ch += 2) {
         uint32_t r[32];
@@ -554,7 +561,7 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
 #pragma unroll
         for (int j = 0; j < 32; ++j) staging[j * GEMM_BM + m] = __uint_as_float(r[j]);
         named_bar_sync(wbar, 128);
-        epi_dispatch<BN>(g.epi, s_ea, staging, m_tile, n_tile, ch, wt, tpos, tkvr, trs_e, wbar);
+        epi_dispatch<BN>(g.epi, s_ea, staging, m_tile, n_tile, ch, wt, tpos, tkvr, trs_e);
         named_bar_sync(wbar, 128);
       }
       tc_fence_before();
@@ -578,7 +585,7 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
         tmem_ld_wait();
         ws_reduce_chunk_own(p.ws, part_slot, parts, own, r, ch, m, staging);
         named_bar_sync(wbar, 128);
-        epi_dispatch<BN>(g.epi, s_ea, staging, m_tile, n_tile, ch, wt, tpos, tkvr, trs_e, wbar);
+        epi_dispatch<BN>(g.epi, s_ea, staging, m_tile, n_tile, ch, wt, tpos, tkvr, trs_e);
         named_bar_sync(wbar, 128);
       }
       tc_fence_before();
@@ -607,7 +614,7 @@ __device__ __forceinline__ bool gemm_epi_phase(const FwdParams& p, int gi, int p
       for (int ch = wg; ch < nch; ch += 2) {
         ws_reduce_chunk<1>(p.ws, part_slot, parts, ch, m, staging);
         named_bar_sync(wbar, 128);
-        epi_dispatch<BN>(g.epi, s_ea, staging, m_tile, n_tile, ch, wt, tpos, tkvr, trs_e, wbar);
+        epi_dispatch<BN>(g.epi, s_ea, staging, m_tile, n_tile, ch, wt, tpos, tkvr, trs_e);
         named_bar_sync(wbar, 128);
       }
     }

@@ -258,6 +258,40 @@ __device__ __forceinline__ void epi_resnorm(const GemmArgs& a, float* st, int m_
   resnorm_store<NJ>(a, sb, m_tile, tok0, j0, nv, ep_tid);
 }
 
+// EPI_RESNORM of one warpgroup's half (tokens 16 half .. 16 half + 15 of every chunk) of a whole tile
+// whose accumulator is in TMEM (tb): epi_resnorm<16>'s arithmetic, the residual read a chunk ahead.  128
+// threads (wt; TMEM lane = tile row m); st: the warpgroup's staging buffer.
+// Latency-bound (residual loads, then the partial sums' chain, per chunk).
+__device__ __forceinline__ void whole_resnorm_half(const GemmArgs& a, uint32_t tb, int nch, int half, int m_tile,
+                                                   int tile_tok0, int wt, int m, float* st, int bar) {
+  constexpr int SR = GEMM_BM + 4;
+  const int row = m_tile * GEMM_BM + m;
+  const bool in = row < a.M;
+  float old[16];
+  auto load_old = [&](int ch) {
+    const int tok = tile_tok0 + ch * 32 + 16 * half, nv = min(16, a.T - tok);
+    const float* base = a.out_f32 + (size_t)tok * a.ldo + row;
+#pragma unroll
+    for (int n = 0; n < 16; ++n) old[n] = (in && n < nv) ? __ldcg(base + (size_t)n * a.ldo) : 0.f;
+  };
+  load_old(0);
+#pragma unroll 1
+  for (int ch = 0; ch < nch; ++ch) {
+    const int tok = tile_tok0 + ch * 32 + 16 * half, nv = min(16, a.T - tok);
+    if (nv <= 0) break;   // (the last chunk's second half may hold no token)
+    uint32_t r[16];
+    tmem_ld_32x32b_x16(tb + ch * 32 + 16 * half, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int n = 0; n < 16; ++n) st[n * SR + m] = in ? old[n] + __uint_as_float(r[n]) : 0.f;
+    if (ch + 1 < nch) load_old(ch + 1);
+    named_bar_sync(bar, 128);
+    if (a.ssq_out != nullptr) resnorm_ssq<16, SR>(a, st, m_tile, tok, 0, nv, wt);
+    resnorm_store<16, SR>(a, st, m_tile, tok, 0, nv, wt);
+    named_bar_sync(bar, 128);
+  }
+}
+
 // Split-K sum (in k order, from zero) of tokens 16 half .. 16 half + 15 of chunk ch of the parts in
 // `slot`, then EPI_RESNORM of those tokens: epi_resnorm<16>'s arithmetic, with the residual loads
 // issued together with the first parts' loads.  PB parts in flight at once.
