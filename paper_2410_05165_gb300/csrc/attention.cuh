@@ -55,4 +55,8 @@ bool attn_make_maps(const __nv_bfloat16* k_cache, const __half* v_cache, int row
 
 cudaError_t attn_launch(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t st, bool pdl);
 
+// The same for one user in one kernel: the tile's visible pages over a cluster of S CTAs (1, 2 or 4; the
+// user's user_splits entry), no partials in global memory.  a.direct: S = 1 and no path keys.
+cudaError_t attn_cluster_launch(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, int S, cudaStream_t st);
+
 }  // namespace atspeed

@@ -87,12 +87,17 @@ struct AttCfg {
 // (count 1); par: bit b is the parity of buffer b's next fill (zero at first), kept identically by
 // every thread from item to item.  Writes the normalised output (a.direct) or the split's
 // unnormalised partials.  Returns false if a bounded wait timed out.
+// Sink::kCustom: the split's share of the tile's visible pages is balanced over user_splits, and the
+// partials go to sink(o, m, l of the thread's two rows) instead (both known at compile time).
 // D - 1 copies are in flight ahead of the arithmetic: a step of 32 keys takes ~0.5 us of tensor and
 // softmax work, a copy 1.5 - 2 us (more from DRAM), so two buffers left the warps waiting for copies.
-template <int HD, int D>
+struct AttGlobalSink {
+  static constexpr bool kCustom = false;
+};
+template <int HD, int D, class Sink = AttGlobalSink>
 __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtensorMap* mv, int tile, int h, int split,
                           uint8_t* smem, uint64_t* bars, uint32_t& par, int tid, int bar_id,
-                          unsigned long long* tr = nullptr, size_t trs = 0) {
+                          unsigned long long* tr = nullptr, size_t trs = 0, const Sink& sink = Sink()) {
 #define ATT_TR(k) do { if (tr && tid == 0) tr[(size_t)(k) * trs] = globaltimer_ns(); } while (0)
   using C = AttCfg<HD, D>;
   constexpr int NDT = HD / 8;    // dim n-tiles of O
@@ -113,7 +118,10 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
   constexpr int BOXW = HD >= 64 ? 64 : HD;
   const int nch = (a.qt_vis[tile] + ATT_PAGE - 1) / ATT_PAGE;
   int c0 = 0, c1 = nch;
-  if (a.chunks_per_split > 0) {
+  if constexpr (Sink::kCustom) {
+    c0 = split * nch / S_u;
+    c1 = (split + 1) * nch / S_u;
+  } else if (a.chunks_per_split > 0) {
     c0 = min(nch, split * a.chunks_per_split);
     c1 = min(nch, c0 + a.chunks_per_split);
   }
@@ -337,6 +345,10 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
   l_b += __shfl_xor_sync(0xffffffffu, l_b, 1);
   l_b += __shfl_xor_sync(0xffffffffu, l_b, 2);
 
+  if constexpr (Sink::kCustom) {
+    sink(o, m_a, l_a, m_b, l_b);
+    return true;
+  }
   if (a.direct) {
     const float ia = l_a > 0.f ? 1.f / l_a : 0.f, ib = l_b > 0.f ? 1.f / l_b : 0.f;
 #pragma unroll

@@ -157,8 +157,10 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
   if (head_dim != 32 && head_dim != 64 && head_dim != 128) return ATSPEED_E_SHAPE;
   cudaStream_t st = (cudaStream_t)stream;
   const int pages = (P + ATT_PAGE - 1) / ATT_PAGE;
-  const int S = std::max(1, (pages + 1) / 2);
   const int nqt = (T + ATT_QTILE - 1) / ATT_QTILE;
+  // CTAs per (query tile, head): about two per SM in all (three fit), no more than pages to share
+  const long long pairs = (long long)nqt * n_heads, want = 2LL * current_grid();
+  const int S = pairs >= want || pages < 2 ? 1 : 2 * pairs >= want || pages < 4 ? 2 : 4;
   for (int p = 0; p < pages; ++p)
     if (h_pages[p] < 0 || (h_pages[p] + 1) * ATT_PAGE > cache_rows) return ATSPEED_E_ARG;
   for (int t = 0; t < T; ++t) {
@@ -168,9 +170,7 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
     for (int j = 0; j < np; ++j)
       if (h_path_rows[t * 4 + j] < 0 || h_path_rows[t * 4 + j] >= cache_rows) return ATSPEED_E_ARG;
   }
-  float* part_o = static_cast<float*>(d_part);
-  float* part_ml = part_o + (size_t)S * T * n_heads * head_dim;
-  int* ip = reinterpret_cast<int*>(part_ml + (size_t)S * T * n_heads * 2);
+  int* ip = static_cast<int*>(d_part);
   std::vector<int> host(4 * nqt + 7 * T + pages + 1, 0);
   int* qt0 = host.data();
   int* qtn = qt0 + nqt;
@@ -187,7 +187,9 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
     qtn[i] = std::min(ATT_QTILE, T - i * ATT_QTILE);
     qtu[i] = 0;
   }
+  bool any_path = false;
   for (int t = 0; t < T; ++t) {
+    any_path |= h_n_path && h_n_path[t] > 0;
     tv[t] = h_vis[t];
     qtv[t / ATT_QTILE] = std::max(qtv[t / ATT_QTILE], h_vis[t]);
     ann[t] = h_n_path ? h_n_path[t] : 0;
@@ -224,14 +226,12 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
   a.page_table = ip + off_pg;
   a.max_pages = std::max(1, pages);
   a.user_splits = ip + off_sp;
-  a.chunks_per_split = 2;
+  a.chunks_per_split = 0;
   a.max_splits = S;
   a.out = static_cast<__nv_bfloat16*>(d_out);
-  a.part_o = part_o;
-  a.part_ml = part_ml;
-  a.direct = false;
+  a.direct = S == 1 && !any_path;
   a.err = nullptr;
-  const cudaError_t e = attn_launch(a, mk, mv, st, false);
+  const cudaError_t e = attn_cluster_launch(a, mk, mv, S, st);
   return e == cudaSuccess ? ATSPEED_OK : ATSPEED_E_CUDA;
 }
 

@@ -88,3 +88,40 @@ def test_rmsnorm_paths(ats, T, d, pad):
     # half a bf16 unit in the last place of the exact value, and fp32 rounding before it
     assert bool(((x[:, :d].double() - ref).abs() <= (2.0 ** -8 + 1e-6) * ref.abs() + 1e-30).all())
     assert bool((x[:, d:] == 7).all())
+
+
+# clusters of 4 (few tiles), 2 and 1 (enough tiles and heads), fewer pages than CTAs, no history at all, queries
+# that see part of it, with and without path keys (one kernel writes its rows directly)
+@pytest.mark.parametrize("H,hd,P,T,paths", [(4, 32, 256, 1, True), (2, 64, 1000, 130, True), (3, 128, 64, 17, True),
+                                            (5, 64, 128, 63, False), (32, 128, 200, 330, True), (40, 32, 300, 250, True),
+                                            (32, 64, 130, 650, True), (32, 128, 321, 641, False), (2, 32, 0, 5, True),
+                                            (1, 128, 2100, 64, True), (80, 32, 70, 257, False)])
+def test_attention_paths(ats, H, hd, P, T, paths):
+    rng = np.random.default_rng(H + P + T)
+    d, n = H * hd, (P + 63) // 64
+    pages = rng.permutation(n + 3)[:n]
+    rows = 64 * (n + 3) + 40
+    q, kc = _randn((T, d), T), _randn((rows, d), P)
+    vc = _randn((rows, d), P + 1).to(torch.float16)
+    vis = np.where(rng.random(T) < 0.5, P, rng.integers(0, P + 1, size=T)).astype(np.int32)
+    n_path = rng.integers(0, 5, size=T).astype(np.int32) if paths else None
+    path = rng.integers(0, rows, size=(T, 4)).astype(np.int32) if paths else None
+    out = ats.op_attention(q, kc, vc, H, hd, P, pages, vis, path, n_path).double().reshape(T, H, hd)
+    prefix = torch.from_numpy((64 * pages[:, None] + np.arange(64)).reshape(-1)[:P].astype(np.int64)).cuda()
+    heads = lambda t: t.double().reshape(-1, H, hd)   # noqa: E731
+    s = torch.einsum("thd,khd->htk", heads(q), heads(kc[prefix]))
+    s = s.masked_fill(~(torch.arange(P)[None, :] < torch.from_numpy(vis)[:, None]).cuda(), float("-inf"))
+    v = heads(vc[prefix])
+    num_v, num_a = [v.transpose(0, 1)], [v.abs().transpose(0, 1)]
+    if paths:
+        pk, pv = [heads(c[torch.from_numpy(path.astype(np.int64)).cuda().reshape(-1)]).reshape(T, 4, H, hd) for c in (kc, vc)]
+        sp = torch.einsum("thd,tjhd->htj", heads(q), pk)
+        sp = sp.masked_fill(~(torch.arange(4)[None, :] < torch.from_numpy(n_path)[:, None]).cuda(), float("-inf"))
+        s = torch.cat([s, sp], 2)
+    w = torch.nan_to_num(torch.softmax(s / hd ** 0.5, 2))   # no key at all: zero
+    ref, mag = [torch.einsum("htk,hkd->thd", w[:, :, :P], x[0]) for x in (num_v, num_a)]
+    if paths:
+        ref = ref + torch.einsum("htj,tjhd->thd", w[:, :, P:], pv)
+        mag = mag + torch.einsum("htj,tjhd->thd", w[:, :, P:], pv.abs())
+    # the weights are rounded to fp16 (2^-11), the result to bf16
+    assert bool(((out - ref).abs() <= 2.0 ** -8 * ref.abs() + 2.0 ** -11 * mag + 1e-5).all())
