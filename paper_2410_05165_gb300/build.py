@@ -18,7 +18,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libatspeed.so")
 
-SOURCES = ["api.cu", "ops.cu", "gemm.cu", "gemm_cluster.cu", "attention.cu", "norm.cu", "select.cu", "tree_ops.cu", "fwd.cu"]
+SOURCES = ["api.cu", "ops.cu", "gemm.cu", "gemm_cluster.cu", "gemm_pair.cu", "attention.cu", "norm.cu", "select.cu", "tree_ops.cu", "fwd.cu"]
 EXTRA = {}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC,

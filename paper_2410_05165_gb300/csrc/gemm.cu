@@ -442,7 +442,7 @@ int gemm_max_tiles() { return MAX_TILES; }
 int gemm_grid_size(int device) {
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-  return sms > 0 ? sms : 1;
+  return sms > 1 ? sms & ~1 : 2;   // whole CTA pairs
 }
 
 cudaError_t gemm_check(const GemmArgs& a, int max_tiles, char* eb, size_t el) {

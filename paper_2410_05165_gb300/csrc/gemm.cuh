@@ -96,4 +96,10 @@ bool gemm_cluster_fits(const GemmArgs& a, int sms);
 cudaError_t gemm_cluster_launch(const GemmArgs& a, unsigned int* err, int sms, cudaStream_t stream, char* errbuf,
                                 size_t errlen);
 
+// The GEMM with many tiles and more than one token tile (gemm_pair.cu): EPI_F32, EPI_RESID, EPI_SWIGLU and
+// EPI_LSE on a grid of `grid` CTAs (gemm_grid_size).
+bool gemm_pair_fits(const GemmArgs& a, int grid);
+cudaError_t gemm_pair_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaStream_t stream, char* errbuf,
+                             size_t errlen);
+
 }  // namespace atspeed

@@ -511,6 +511,27 @@ __device__ __forceinline__ void epi_chunk(const GemmArgs& a, const float* st, in
   }
 }
 
+// EPI_F32 / EPI_RESID of 32 tokens from tok0 held by a thread that owns weight row `row` (r: the
+// accumulator's 32 columns): per token a warp stores 32 consecutive values.
+template <int EPI>
+__device__ __forceinline__ void epi_rows(const GemmArgs& a, const uint32_t (&r)[32], int row, int tok0) {
+  if (row >= a.M) return;
+  const int nv = min(32, a.T - tok0);
+  float* o = a.out_f32 + (size_t)tok0 * a.ldo + row;
+  if constexpr (EPI == EPI_RESID) {
+    float old[32];
+#pragma unroll
+    for (int n = 0; n < 32; ++n) old[n] = n < nv ? __ldcg(o + (size_t)n * a.ldo) : 0.f;
+#pragma unroll
+    for (int n = 0; n < 32; ++n)
+      if (n < nv) o[(size_t)n * a.ldo] = old[n] + __uint_as_float(r[n]);
+  } else {
+#pragma unroll
+    for (int n = 0; n < 32; ++n)
+      if (n < nv) o[(size_t)n * a.ldo] = __uint_as_float(r[n]);
+  }
+}
+
 // ---- split-K partials (stream-K tiles shared by several CTAs)
 // A workspace slot holds one CTA's fp32 partial of a 128-row tile for up to 256 tokens, laid out
 // [token/4][row][4] so that a thread (one weight row) moves four tokens per 16-byte access.

@@ -52,7 +52,7 @@ atspeed_status run_gemm(cudaStream_t st, const GemmArgs& a, void* ws) {
   const int grid = current_grid();
   const GemmScratch s = scratch_from(ws);
   if (gemm_cluster_fits(a, grid)) return gemm_status(gemm_cluster_launch(a, s.err, grid, st, eb, sizeof eb));
-  return gemm_status(gemm_launch(a, s, grid, st, false, eb, sizeof eb));
+  return gemm_status(gemm_pair_launch(a, s, grid, st, eb, sizeof eb));
 }
 
 // ---------------------------------------------------------------------------------------------
