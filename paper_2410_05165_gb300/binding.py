@@ -340,8 +340,8 @@ def op_workspace(device: int = 0) -> torch.Tensor:
 def op_gemm(W: torch.Tensor, X: torch.Tensor, T: int, Y: Optional[torch.Tensor] = None, accumulate=False,
             stream=None) -> torch.Tensor:
     M, K = W.shape
-    if Y is None:
-        Y = torch.zeros(T, M, dtype=torch.float32, device=W.device)
+    if Y is None:   # (every value is written unless it is added to)
+        Y = (torch.zeros if accumulate else torch.empty)(T, M, dtype=torch.float32, device=W.device)
     _check(load().atspeed_op_gemm(_stream(stream), W.data_ptr(), X.data_ptr(), M, K, T, X.shape[0], Y.data_ptr(),
                                   Y.shape[1], 1 if accumulate else 0, op_workspace().data_ptr()))
     return Y
@@ -351,8 +351,8 @@ def op_gemm_noalloc(W: torch.Tensor, X: torch.Tensor, T: int, Y: Optional[torch.
                     stream=None) -> torch.Tensor:
     """atspeed_op_gemm without a workspace argument (the library's fixed scratch array is used)."""
     M, K = W.shape
-    if Y is None:
-        Y = torch.zeros(T, M, dtype=torch.float32, device=W.device)
+    if Y is None:   # (every value is written unless it is added to)
+        Y = (torch.zeros if accumulate else torch.empty)(T, M, dtype=torch.float32, device=W.device)
     _check(load().atspeed_op_gemm_noalloc(_stream(stream), W.data_ptr(), X.data_ptr(), M, K, T, X.shape[0],
                                           Y.data_ptr(), Y.shape[1], 1 if accumulate else 0))
     return Y
@@ -367,7 +367,7 @@ def op_status(noalloc: bool = False, stream=None) -> int:
 
 def op_gemm_swiglu(W: torch.Tensor, X: torch.Tensor, T: int, stream=None) -> torch.Tensor:
     F2, K = W.shape
-    out = torch.zeros(T, F2 // 2, dtype=torch.bfloat16, device=W.device)
+    out = torch.empty(T, F2 // 2, dtype=torch.bfloat16, device=W.device)
     _check(load().atspeed_op_gemm_swiglu(_stream(stream), W.data_ptr(), X.data_ptr(), F2 // 2, K, T, X.shape[0],
                                          out.data_ptr(), out.shape[1], op_workspace().data_ptr()))
     return out
@@ -375,7 +375,7 @@ def op_gemm_swiglu(W: torch.Tensor, X: torch.Tensor, T: int, stream=None) -> tor
 
 def op_rmsnorm(h: torch.Tensor, g: torch.Tensor, eps: float, stream=None) -> torch.Tensor:
     T, d = h.shape
-    x = torch.zeros(T, d, dtype=torch.bfloat16, device=h.device)
+    x = torch.empty(T, d, dtype=torch.bfloat16, device=h.device)
     _check(load().atspeed_op_rmsnorm(_stream(stream), h.data_ptr(), g.data_ptr(), T, d, eps, x.data_ptr(), d))
     return x
 
@@ -385,15 +385,15 @@ def op_attention(q: torch.Tensor, kc: torch.Tensor, vc: torch.Tensor, n_heads: i
                  n_path: Optional[Sequence[int]] = None, stream=None) -> torch.Tensor:
     lib = load()
     T = q.shape[0]
-    out = torch.zeros(T, n_heads * head_dim, dtype=torch.bfloat16, device=q.device)
+    out = torch.empty(T, n_heads * head_dim, dtype=torch.bfloat16, device=q.device)
     scratch = torch.empty(lib.atspeed_op_attention_scratch(T, n_heads, head_dim, P), dtype=torch.uint8,
                           device=q.device)
-    pg, pgp = _i32(list(pages) if len(pages) else [0])
+    pg, pgp = _i32(pages if len(pages) else [0])
     vv, vvp = _i32(vis)
-    pr = np.zeros((T, 4), np.int32) if path_rows is None else path_rows
-    pr, prp = _i32(pr)
-    npth = np.zeros(T, np.int32) if n_path is None else n_path
-    npth, npp = _i32(npth)
+    pr = prp = npth = npp = None   # (no counts: no path keys, and nothing to pass)
+    if n_path is not None:
+        pr, prp = _i32(np.zeros((T, 4), np.int32) if path_rows is None else path_rows)
+        npth, npp = _i32(n_path)
     _check(lib.atspeed_op_attention(_stream(stream), q.data_ptr(), kc.data_ptr(), vc.data_ptr(), kc.shape[0], T,
                                     n_heads, head_dim, P, pgp, vvp, prp, npp, out.data_ptr(), scratch.data_ptr()))
     return out

@@ -90,7 +90,8 @@ struct ModelRt {
   int lse_ld = 0;
   bf16* root_x = nullptr;
   int root_rows = 0;
-  // per-token forward inputs
+  // per-token forward inputs (pos, kvrow, tuser, tvis: consecutive sections of tok_blk)
+  int* tok_blk = nullptr;
   int *tok = nullptr, *pos = nullptr, *kvrow = nullptr, *tuser = nullptr, *tvis = nullptr, *anc = nullptr,
       *ancn = nullptr;
   int *qt_t0 = nullptr, *qt_n = nullptr, *qt_user = nullptr, *qt_vis = nullptr, *rows_sel = nullptr,
@@ -305,6 +306,14 @@ void carve_nodes(atspeed_ctx* c, size_t n, int B, int g) {
 constexpr size_t NODE_INTS = 21;   // ints per slot in the node table (the n_* arrays above)
 size_t o_blk_ints(int mu, int mK) { return 4 * (size_t)mu + 15 * (size_t)mu * mK; }
 
+// Points a model's pos, kvrow, tuser and tvis at consecutive sections of T ints of their block.
+void carve_token_tables(ModelRt& m, int T) {
+  m.pos = m.tok_blk;
+  m.kvrow = m.pos + T;
+  m.tuser = m.kvrow + T;
+  m.tvis = m.tuser + T;
+}
+
 void init_model(atspeed_ctx* c, ModelRt& m, const atspeed_model_desc* md, const char* name) {
   if (!md) return;
   if (md->n_layers <= 0 || md->d_model <= 0 || md->n_heads <= 0 || md->d_ffn <= 0 || md->vocab <= 0) {
@@ -404,10 +413,8 @@ void alloc_model(atspeed_ctx* c, ModelRt& m) {
   m.root_rows = ((L.max_users + 255) / 256) * 256;
   m.root_x = dalloc<bf16>(c, (size_t)m.root_rows * m.d);
   m.tok = dalloc<int>(c, m.Tcap);
-  m.pos = dalloc<int>(c, m.Tcap);
-  m.kvrow = dalloc<int>(c, m.Tcap);
-  m.tuser = dalloc<int>(c, m.Tcap);
-  m.tvis = dalloc<int>(c, m.Tcap);
+  m.tok_blk = dalloc<int>(c, 4 * (size_t)m.Tcap);
+  carve_token_tables(m, m.Tcap);
   m.anc = dalloc<int>(c, (size_t)m.Tcap * 4);
   m.ancn = dalloc<int>(c, m.Tcap);
   const int max_qt = m.Tcap / ATT_QTILE + L.max_users + 1;
@@ -906,6 +913,7 @@ void forward_nodes(atspeed_ctx* c, ModelRt& m, bool target, const std::vector<in
   const int T = (int)nodes.size();
   const TreeDev t = tree_dev(c);
   upload(c, st, c->fwd_nodes, nodes.data(), (size_t)T * 4);
+  carve_token_tables(m, T);
   FwdTokens f{m.tok, m.pos, m.kvrow, m.tuser, m.tvis, m.anc, m.ancn};
   CK(tree_gather_launch(t, c->fwd_nodes, T, c->u_P, c->code_base, target, row_base, f, st, c->pdl));
   c->n_launch += 1;
@@ -1272,7 +1280,8 @@ void prefill_impl(atspeed_ctx* c, cudaStream_t st, int n_users, const int32_t* d
   c->B = n_users;
   c->users.assign(n_users, UserState{});
   const int T = h_off[n_users] - h_off[0];
-  std::vector<int> pos(T), kvrow(T), tuser(T), tvis(T);
+  std::vector<int> tables(4 * (size_t)T);   // pos, kvrow, tuser, tvis of every token: one upload per model
+  int *pos = tables.data(), *kvrow = pos + T, *tuser = kvrow + T, *tvis = tuser + T;
   FwdPlan p;
   p.T = T;
   p.prefill = true;
@@ -1303,10 +1312,8 @@ void prefill_impl(atspeed_ctx* c, cudaStream_t st, int n_users, const int32_t* d
   p.logit_row_base = 0;
   for (ModelRt* m : {&c->tgt, &c->drf}) {
     if (!m->present) continue;
-    upload(c, st, m->pos, pos.data(), (size_t)T * 4);
-    upload(c, st, m->kvrow, kvrow.data(), (size_t)T * 4);
-    upload(c, st, m->tuser, tuser.data(), (size_t)T * 4);
-    upload(c, st, m->tvis, tvis.data(), (size_t)T * 4);
+    carve_token_tables(*m, T);
+    upload(c, st, m->tok_blk, tables.data(), tables.size() * sizeof(int));
     forward(c, *m, p, st);
     // the last history tokens' final-norm rows, for a FULL-normalised first step
     CK(cudaMemcpyAsync(m->root_x, m->x, (size_t)n_users * m->d * sizeof(bf16), cudaMemcpyDeviceToDevice, st));
@@ -1524,8 +1531,10 @@ atspeed_status atspeed_create(const atspeed_model_desc* target, const atspeed_mo
     c->u_step = c->u_blk + 2 * mu;
     c->u_P = c->u_blk + 3 * mu;
     c->fwd_nodes = dalloc<int>(c, nn);
-    // staging: the largest per-step upload is the node table; forward plans and outputs are small
-    c->stage_cap = 2 * (NODE_INTS * nn + n_cnt_max) * sizeof(int) + ((size_t)1 << 20);
+    // staging: the largest uploads are the node table and a prefill's token tables; forward plans and
+    // outputs are small
+    c->stage_cap = 2 * (NODE_INTS * nn + n_cnt_max) * sizeof(int) + ((size_t)1 << 20) +
+                   4 * (size_t)mu * lim->max_prompt * sizeof(int);
     {
       void* hp = nullptr;
       CK(cudaMallocHost(&hp, c->stage_cap));
@@ -1874,22 +1883,18 @@ atspeed_status atspeed_set_tree(atspeed_ctx* c, atspeed_stream stream, int n_lev
     }
     const int K = c->step_K, N = c->step_N, G = c->step_gamma, stride = K + G * N, W = c->lim.max_N;
     const size_t n = (size_t)c->B * stride;
-    std::vector<int> code(n), prank(n), trie(n), path(n * 4), rt(n), rd(n), at(n * 4), ad(n * 4), lgd(n),
-        cnt((size_t)c->B * (G + 1));
-    std::vector<float> sq(n), sp(n);
+    // the node table comes back, is edited and goes out again as the one block it is (carve_nodes)
+    const size_t ntab = NODE_INTS * n + (size_t)c->B * (G + 1);
     stage_sync(c, st);
-    CK(cudaMemcpy(code.data(), c->n_code, n * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(trie.data(), c->n_trie, n * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(path.data(), c->n_path, n * 16, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(rt.data(), c->n_row_t, n * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(rd.data(), c->n_row_d, n * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(at.data(), c->n_anc_t, n * 16, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(ad.data(), c->n_anc_d, n * 16, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(lgd.data(), c->n_lg_d, n * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(sq.data(), c->n_sq, n * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(sp.data(), c->n_sp, n * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(prank.data(), c->n_prank, n * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(cnt.data(), c->n_cnt, cnt.size() * 4, cudaMemcpyDeviceToHost));
+    int* const tab = stage_alloc<int>(c, st, ntab);
+    CK(cudaMemcpyAsync(tab, c->n_blk, ntab * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    const auto at_host = [&](const void* dev) { return tab + (static_cast<const int*>(dev) - c->n_blk); };
+    int *const code = at_host(c->n_code), *const prank = at_host(c->n_prank), *const trie = at_host(c->n_trie),
+        *const path = at_host(c->n_path), *const rt = at_host(c->n_row_t), *const rd = at_host(c->n_row_d),
+        *const at = at_host(c->n_anc_t), *const ad = at_host(c->n_anc_d), *const lgd = at_host(c->n_lg_d),
+        *const cnt = at_host(c->n_cnt);
+    float *const sq = reinterpret_cast<float*>(at_host(c->n_sq)), *const sp = reinterpret_cast<float*>(at_host(c->n_sp));
     int drow = c->B;  // draft logits rows for injected parents
     std::vector<float> dl;
     std::vector<int> dl_rows;
@@ -1961,16 +1966,7 @@ atspeed_status atspeed_set_tree(atspeed_ctx* c, atspeed_stream stream, int n_lev
       }
       CK(cudaMemcpy(m.logits + (size_t)c->B * ITEM_ROWS, dl.data(), dl.size() * 4, cudaMemcpyHostToDevice));
     }
-    CK(cudaMemcpy(c->n_code, code.data(), n * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->n_prank, prank.data(), n * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->n_trie, trie.data(), n * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->n_path, path.data(), n * 16, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->n_anc_t, at.data(), n * 16, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->n_anc_d, ad.data(), n * 16, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->n_lg_d, lgd.data(), n * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->n_sq, sq.data(), n * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->n_sp, sp.data(), n * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->n_cnt, cnt.data(), cnt.size() * 4, cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(c->n_blk, tab, ntab * sizeof(int), cudaMemcpyHostToDevice, st));
     c->levels_done = n_levels;
     c->tree_injected = true;
     upload_users(c, st);
