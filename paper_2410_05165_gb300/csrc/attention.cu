@@ -42,7 +42,7 @@ template <int HD>
 __global__ void __launch_bounds__(128) attn_combine_kernel(const AttnArgs a) {
   pdl_launch_dependents();
   pdl_wait();
-  attn_combine_group<HD>(a, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x);
+  attn_combine_group<HD>(a, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, []() { return true; });
 }
 
 // ---- the operator's attention: one kernel, the prefix splits of a (query tile, head) in one cluster

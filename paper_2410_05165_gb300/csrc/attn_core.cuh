@@ -394,8 +394,10 @@ constexpr int ATT_CQ = 16;
 // HD / 8 consecutive dimensions; a path-key dot product adds the eight partial sums by a butterfly
 // over the eight lanes (exact in any lane, as fp32 addition commutes), so the result does not
 // depend on the schedule that calls it.
-template <int HD>
-__device__ void attn_combine_group(const AttnArgs& a, int tile, int h, int qg, int ctid) {
+// wait(): called once the path-key scores, which need nothing from the splits, are there; returns whether
+// every split's partials are published (false: give up).
+template <int HD, class Wait>
+__device__ __forceinline__ bool attn_combine_group(const AttnArgs& a, int tile, int h, int qg, int ctid, Wait wait) {
   constexpr int TPQ = 8, DH = HD / TPQ;
   const int ql = qg * ATT_CQ + (ctid >> 3), part = ctid & 7;
   const int t0 = a.qt_t0[tile], nq = a.qt_n[tile];
@@ -418,38 +420,57 @@ __device__ void attn_combine_group(const AttnArgs& a, int tile, int h, int qg, i
   int arow[ATT_MAX_ANC];
 #pragma unroll
   for (int j = 0; j < ATT_MAX_ANC; ++j) arow[j] = j < na ? a.anc_row[t * ATT_MAX_ANC + j] : 0;
-  float M = -INFINITY;
-  for (int s = 0; s < S; ++s) M = fmaxf(M, __ldcg(a.part_ml + (((size_t)s * a.T + t) * a.n_heads + h) * 2));
   // path keys (rows written earlier in this forward; cached loads, queries share ancestors)
   float sa[ATT_MAX_ANC];
+  __nv_bfloat16 kb[ATT_MAX_ANC][DH];
+#pragma unroll
+  for (int j = 0; j < ATT_MAX_ANC; ++j)
+#pragma unroll
+    for (int i = 0; i < DH; i += 4)
+      *reinterpret_cast<uint2*>(kb[j] + i) = *reinterpret_cast<const uint2*>(a.k_cache + (size_t)arow[j] * d + dim0 + i);
 #pragma unroll
   for (int j = 0; j < ATT_MAX_ANC; ++j) {
     float pd = 0.f;
-    if (j < na) {
-      __nv_bfloat16 kb[DH];
 #pragma unroll
-      for (int i = 0; i < DH; i += 4)
-        *reinterpret_cast<uint2*>(kb + i) = *reinterpret_cast<const uint2*>(a.k_cache + (size_t)arow[j] * d + dim0 + i);
-#pragma unroll
-      for (int i = 0; i < DH; ++i) pd += qv[i] * __bfloat162float(kb[i]);
-    }
+    for (int i = 0; i < DH; ++i) pd += qv[i] * __bfloat162float(kb[j][i]);
     pd += __shfl_xor_sync(0xffffffffu, pd, 1);
     pd += __shfl_xor_sync(0xffffffffu, pd, 2);
     pd += __shfl_xor_sync(0xffffffffu, pd, 4);
     sa[j] = pd * scale;
-    if (j < na) M = fmaxf(M, sa[j]);
   }
+  if (!wait()) return false;
+  float M = -INFINITY;
+  for (int s0 = 0; s0 < S; s0 += 4) {
+    float mv[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      mv[i] = s0 + i < S ? __ldcg(a.part_ml + (((size_t)(s0 + i) * a.T + t) * a.n_heads + h) * 2) : -INFINITY;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) M = fmaxf(M, mv[i]);
+  }
+#pragma unroll
+  for (int j = 0; j < ATT_MAX_ANC; ++j)
+    if (j < na) M = fmaxf(M, sa[j]);
   const float Mu = (M == -INFINITY) ? 0.f : M;
   float L = 0.f, o[DH];
 #pragma unroll
   for (int i = 0; i < DH; ++i) o[i] = 0.f;
+  const size_t bs = (size_t)a.T * a.n_heads;
+  float2 ml_n;
+  float4 pv_n[DH / 4];
+  auto load_part = [&](int s) {
+    const size_t b = (size_t)s * bs + (size_t)t * a.n_heads + h;
+    ml_n = __ldcg(reinterpret_cast<const float2*>(a.part_ml + b * 2));
+#pragma unroll
+    for (int i = 0; i < DH / 4; ++i) pv_n[i] = __ldcg(reinterpret_cast<const float4*>(a.part_o + b * HD + part * DH) + i);
+  };
+  load_part(0);
   for (int s = 0; s < S; ++s) {
-    const size_t b = ((size_t)s * a.T + t) * a.n_heads + h;
-    const float2 ml = __ldcg(reinterpret_cast<const float2*>(a.part_ml + b * 2));
-    const float* po = a.part_o + b * HD + part * DH;
+    const float2 ml = ml_n;
     float4 pv[DH / 4];
 #pragma unroll
-    for (int i = 0; i < DH; i += 4) pv[i / 4] = __ldcg(reinterpret_cast<const float4*>(po + i));
+    for (int i = 0; i < DH / 4; ++i) pv[i] = pv_n[i];
+    if (s + 1 < S) load_part(s + 1);
     const float w = exp2f(ml.x - Mu);
     L += ml.y * w;
 #pragma unroll
@@ -460,23 +481,26 @@ __device__ void attn_combine_group(const AttnArgs& a, int tile, int h, int qg, i
       o[i + 3] += pv[i / 4].w * w;
     }
   }
+  __half vb[ATT_MAX_ANC][DH];
+#pragma unroll
+  for (int j = 0; j < ATT_MAX_ANC; ++j)
+#pragma unroll
+    for (int i = 0; i < DH; i += 4)
+      *reinterpret_cast<uint2*>(vb[j] + i) = *reinterpret_cast<const uint2*>(a.v_cache + (size_t)arow[j] * d + dim0 + i);
 #pragma unroll
   for (int j = 0; j < ATT_MAX_ANC; ++j) {
     if (j >= na) continue;
     const float w = exp2f(sa[j] - Mu);
     L += w;
-    __half vb[DH];
 #pragma unroll
-    for (int i = 0; i < DH; i += 4)
-      *reinterpret_cast<uint2*>(vb + i) = *reinterpret_cast<const uint2*>(a.v_cache + (size_t)arow[j] * d + dim0 + i);
-#pragma unroll
-    for (int i = 0; i < DH; ++i) o[i] += w * __half2float(vb[i]);
+    for (int i = 0; i < DH; ++i) o[i] += w * __half2float(vb[j][i]);
   }
-  if (!active) return;
+  if (!active) return true;
   const float inv = L > 0.f ? 1.f / L : 0.f;
 #pragma unroll
   for (int i = 0; i < DH; i += 2)
     *reinterpret_cast<__nv_bfloat162*>(a.out + (size_t)t * d + dim0 + i) = __floats2bfloat162_rn(o[i] * inv, o[i + 1] * inv);
+  return true;
 }
 
 }  // namespace atspeed

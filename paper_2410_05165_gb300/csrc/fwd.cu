@@ -395,17 +395,24 @@ __device__ __forceinline__ bool attn_phase(const FwdParams& p, int l, uint8_t* a
     // one round (2 G work slots), or the awaited ones in a later round, never an earlier one -- then
     // split s merges query groups s, s + S_u, ...  The counter only grows during a launch: layer l
     // completes at S_u * (l + 1).
-    __threadfence();
+    // publish this split's partials (every thread's are stored before the barrier, thread 0's release
+    // carries them); then split s merges query groups s, s + S_u, ... once all splits of (tile, h) are
+    // there -- all items run in one round (2 G work slots), or the awaited ones in a later round, never
+    // an earlier one.  The counter only grows during a launch: layer l completes at S_u * (l + 1).
     named_bar_sync(wbar, 128);
-    if (wt == 0) {
-      int* cnt = &p.att_counters[tile * H + h];
-      atomicAdd(cnt, 1);
-      *flag = counter_wait(cnt, S_u * (l + 1), p.err) ? 1 : 0;
-    }
-    named_bar_sync(wbar, 128);
-    if (!*flag) return false;
+    int* cnt = &p.att_counters[tile * H + h];
+    if (S_u > 1 && wt == 0) red_release_add(cnt, 1);
+    bool waited = S_u == 1;
+    const auto wait = [&]() {
+      if (waited) return true;
+      waited = true;
+      if (wt == 0) *flag = counter_wait(cnt, S_u * (l + 1), p.err) ? 1 : 0;
+      named_bar_sync(wbar, 128);
+      return *flag != 0;
+    };
     const int nq = a.qt_n[tile];
-    for (int qg = split; qg * ATT_CQ < nq; qg += S_u) attn_combine_group<HD>(a, tile, h, qg, wt);
+    for (int qg = split; qg * ATT_CQ < nq; qg += S_u)
+      if (!attn_combine_group<HD>(a, tile, h, qg, wt, wait)) return false;
     named_bar_sync(wbar, 128);
     if (tr_on && wt == 0) p.trace[((size_t)5 * NP + ph) * G + c] = globaltimer_ns();
   }
