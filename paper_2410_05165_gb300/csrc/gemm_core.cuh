@@ -189,12 +189,31 @@ __device__ __forceinline__ void resnorm_ssq(const GemmArgs& a, const float* sr, 
                                             int ep_tid) {
   if (ep_tid < 4 * NJ) {
     const int jj = ep_tid >> 2, sub = ep_tid & 3, j = j0 + jj;
-    const float* sj = sr + jj * SR + sub * 32;
-    float s = ssq32([&](int r) { return sj[r]; }, ssq_rot(sub));
+    // ssq32's order, four values per load (the rotation is a multiple of 8)
+    static_assert(SR % 4 == 0, "16-byte aligned rows");
+    const float4* s4 = reinterpret_cast<const float4*>(sr + jj * SR + sub * 32);
+    float4 x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = s4[(i + (ssq_rot(sub) >> 2)) & 7];
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      s = __fmaf_rn(x[i].x, x[i].x, s);
+      s = __fmaf_rn(x[i].y, x[i].y, s);
+      s = __fmaf_rn(x[i].z, x[i].z, s);
+      s = __fmaf_rn(x[i].w, x[i].w, s);
+    }
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     s += __shfl_xor_sync(0xffffffffu, s, 2);
     if (sub == 0 && jj < nv) a.ssq_out[(size_t)m_tile * a.ssq_ld + tok0 + j] = s;
   }
+}
+
+// The gains of the four rows that a thread stores (resnorm_store), read before the sums so that the
+// stores do not wait for them.
+__device__ __forceinline__ uint2 resnorm_gain(const GemmArgs& a, int m_tile, int ep_tid) {
+  const int row = m_tile * GEMM_BM + 4 * (ep_tid & 31);
+  return a.gain != nullptr && row < a.M ? *reinterpret_cast<const uint2*>(a.gain + row) : make_uint2(0, 0);
 }
 
 // The updated residual of tokens j0 .. j0 + NJ - 1 of a chunk (st, [token][128 rows]; nv of them
@@ -203,19 +222,14 @@ __device__ __forceinline__ void resnorm_ssq(const GemmArgs& a, const float* sr, 
 // 128 rows in one piece.  (M, the residual's width, is a multiple of 4.)
 template <int NJ, int SR = GEMM_BM>
 __device__ __forceinline__ void resnorm_store(const GemmArgs& a, const float* sr, int m_tile, int tok0, int j0, int nv,
-                                              int ep_tid) {
+                                              int ep_tid, uint2 graw) {
   constexpr int TPW = NJ / 4;   // tokens per warp
   const int rq = ep_tid & 31, w = ep_tid >> 5;
   const int row = m_tile * GEMM_BM + 4 * rq;
   if (row >= a.M) return;
   const bool xg = a.gain != nullptr;
-  float2 g01 = make_float2(0.f, 0.f), g23 = g01;
-  if (xg) {
-    const uint2 graw = *reinterpret_cast<const uint2*>(a.gain + row);
-    const __nv_bfloat162* gb = reinterpret_cast<const __nv_bfloat162*>(&graw);
-    g01 = __bfloat1622float2(gb[0]);
-    g23 = __bfloat1622float2(gb[1]);
-  }
+  const __nv_bfloat162* gb = reinterpret_cast<const __nv_bfloat162*>(&graw);
+  const float2 g01 = __bfloat1622float2(gb[0]), g23 = __bfloat1622float2(gb[1]);
 #pragma unroll
   for (int k = 0; k < TPW; ++k) {
     const int n = w * TPW + k;
@@ -247,6 +261,7 @@ __device__ __forceinline__ void epi_resnorm(const GemmArgs& a, float* st, int m_
   const bool in = row < a.M;
   const float* base = a.out_f32 + (size_t)(tok0 + j0) * a.ldo + row;
   float* sb = st + j0 * GEMM_BM;
+  const uint2 graw = resnorm_gain(a, m_tile, ep_tid);
   float old[NJ];
 #pragma unroll
   for (int n = 0; n < NJ; ++n) old[n] = (in && n < nv) ? __ldcg(base + (size_t)n * a.ldo) : 0.f;
@@ -255,7 +270,7 @@ __device__ __forceinline__ void epi_resnorm(const GemmArgs& a, float* st, int m_
   // the sums of squares before the stores (their shared-memory reads would queue behind them)
   named_bar_sync(bar, 128);
   if (a.ssq_out != nullptr) resnorm_ssq<NJ>(a, sb, m_tile, tok0, j0, nv, ep_tid);
-  resnorm_store<NJ>(a, sb, m_tile, tok0, j0, nv, ep_tid);
+  resnorm_store<NJ>(a, sb, m_tile, tok0, j0, nv, ep_tid, graw);
 }
 
 // EPI_RESNORM of one warpgroup's half (tokens 16 half .. 16 half + 15 of every chunk) of a whole tile
@@ -275,6 +290,7 @@ __device__ __forceinline__ void whole_resnorm_half(const GemmArgs& a, uint32_t t
     for (int n = 0; n < 16; ++n) old[n] = (in && n < nv) ? __ldcg(base + (size_t)n * a.ldo) : 0.f;
   };
   load_old(0);
+  const uint2 graw = resnorm_gain(a, m_tile, wt);
 #pragma unroll 1
   for (int ch = 0; ch < nch; ++ch) {
     const int tok = tile_tok0 + ch * 32 + 16 * half, nv = min(16, a.T - tok);
@@ -287,7 +303,7 @@ __device__ __forceinline__ void whole_resnorm_half(const GemmArgs& a, uint32_t t
     if (ch + 1 < nch) load_old(ch + 1);
     named_bar_sync(bar, 128);
     if (a.ssq_out != nullptr) resnorm_ssq<16, SR>(a, st, m_tile, tok, 0, nv, wt);
-    resnorm_store<16, SR>(a, st, m_tile, tok, 0, nv, wt);
+    resnorm_store<16, SR>(a, st, m_tile, tok, 0, nv, wt, graw);
     named_bar_sync(bar, 128);
   }
 }
@@ -304,6 +320,7 @@ __device__ __forceinline__ void ws_reduce_resnorm_half(const GemmArgs& a, const 
   const int m = ep_tid, row = m_tile * GEMM_BM + m;
   const bool in = row < a.M;
   const float* base = a.out_f32 + (size_t)(tok0 + j0) * a.ldo + row;
+  const uint2 graw = resnorm_gain(a, m_tile, ep_tid);
   float old[16], acc[16];
 #pragma unroll
   for (int n = 0; n < 16; ++n) {
@@ -342,7 +359,7 @@ __device__ __forceinline__ void ws_reduce_resnorm_half(const GemmArgs& a, const 
   for (int n = 0; n < 16; ++n) st[n * SR + m] = in ? old[n] + acc[n] : 0.f;
   named_bar_sync(bar, 128);
   if (a.ssq_out != nullptr) resnorm_ssq<16, SR>(a, st, m_tile, tok0, j0, nv, ep_tid);
-  resnorm_store<16, SR>(a, st, m_tile, tok0, j0, nv, ep_tid);
+  resnorm_store<16, SR>(a, st, m_tile, tok0, j0, nv, ep_tid, graw);
 }
 
 // silu(g) * u, silu(g) = g / (1 + e^-g), with the hardware exponential and an approximate divide (a few
