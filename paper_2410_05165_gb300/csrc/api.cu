@@ -617,7 +617,13 @@ void gemm(atspeed_ctx* c, const GemmArgs& a, cudaStream_t st, int kind, int grid
                        : a.epi == EPI_RESNORM ? (a.gain ? 10.0 * a.M : 8.0 * a.M)
                        : a.epi == EPI_SWIGLU ? 1.0 * a.M : 2.0 * a.M;
   ProfScope ps(c, st, kind, 2.0 * a.M * a.K + 2.0 * a.T * a.K + out_b * a.T, 2.0 * a.M * a.K * a.T);
-  cudaError_t e = gemm_launch(a, c->gs, grid, st, c->pdl && !c->prof, eb, sizeof eb);
+  // the whole-vocabulary head takes the operators' kernels and the whole GPU, the forward's GEMMs the
+  // work split they share with the persistent kernel (33024 rows of 4096: 4 tokens 50 -> 45 us, 6.0 TB/s;
+  // 960 tokens 187 -> 162 us, 1.6 PFLOP/s)
+  cudaError_t e = a.epi != EPI_LSE ? gemm_launch(a, c->gs, grid, st, c->pdl && !c->prof, eb, sizeof eb)
+                  : gemm_cluster_fits(a, c->gemm_grid)
+                      ? gemm_cluster_launch(a, c->err_word, c->gemm_grid, st, eb, sizeof eb)
+                      : gemm_pair_launch(a, c->gs, c->gemm_grid, st, eb, sizeof eb);
   c->n_launch += 1;
   if (e != cudaSuccess) {
     set_err(c, "gemm launch failed: %s %s", cudaGetErrorString(e), eb);

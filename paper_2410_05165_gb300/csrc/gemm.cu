@@ -376,7 +376,7 @@ cudaError_t launch_bn(EpiKind e, const CUtensorMap& ma, const CUtensorMap& mb, c
     case EPI_RESID: return launch_t<BN, EPI_RESID>(ma, mb, kp, st, pdl);
     case EPI_SWIGLU: return launch_t<BN, EPI_SWIGLU>(ma, mb, kp, st, pdl);
     case EPI_QKV: return launch_t<BN, EPI_QKV>(ma, mb, kp, st, pdl);
-    case EPI_LSE: return launch_t<BN, EPI_LSE>(ma, mb, kp, st, pdl);
+    case EPI_LSE: break;   // gemm_cluster.cu, gemm_pair.cu
     case EPI_RESNORM: return launch_t<BN, EPI_RESNORM>(ma, mb, kp, st, pdl);
   }
   return cudaErrorInvalidValue;

@@ -90,8 +90,8 @@ cudaError_t gemm_check(const GemmArgs& a, int max_tiles, char* errbuf, size_t er
 cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaStream_t stream, bool pdl,
                         char* errbuf, size_t errlen);
 
-// The operators' GEMM with few output tiles (gemm_cluster.cu): EPI_F32, EPI_RESID and EPI_SWIGLU, no
-// workspace.  gemm_cluster_fits: whether it is the kernel for these sizes on a GPU of `sms` SMs.
+// The operators' GEMM with few output tiles (gemm_cluster.cu): EPI_F32, EPI_RESID, EPI_SWIGLU and EPI_LSE,
+// no workspace.  gemm_cluster_fits: whether it is the kernel for these sizes on a GPU of `sms` SMs.
 bool gemm_cluster_fits(const GemmArgs& a, int sms);
 cudaError_t gemm_cluster_launch(const GemmArgs& a, unsigned int* err, int sms, cudaStream_t stream, char* errbuf,
                                 size_t errlen);

@@ -251,11 +251,39 @@ __global__ void __launch_bounds__(THREADS, 2)
             for (int n = 0; n < GROUP; ++n)
               if (n < nv) o[(size_t)n * a.ldo] = EPI == EPI_RESID ? old[n] + acc[n] : acc[n];
           }
-        } else {   // EPI_SWIGLU: rows 0-63 of the tile are gates, 64-127 the matching ups
-          named_bar_sync(1 + wg, 128);   // the previous group's rows have been read
+          continue;
+        }
+        named_bar_sync(1 + wg, 128);   // the previous group's rows have been read
 #pragma unroll
-          for (int n = 0; n < GROUP; ++n) stg[n * STG_LD + m] = acc[n];
-          named_bar_sync(1 + wg, 128);
+        for (int n = 0; n < GROUP; ++n) stg[n * STG_LD + m] = acc[n];
+        named_bar_sync(1 + wg, 128);
+        if constexpr (EPI == EPI_LSE) {
+          // (max, sum of exp(y - max)) of each token over the tile's rows: eight threads per token, 16 rows
+          // each (four at a time), then combined in a fixed order
+          const int j = wt >> 3, sub = wt & 7;
+          const int valid = min(GEMM_BM, a.M - m_tile * GEMM_BM) - sub * 16;
+          const float4* s4 = reinterpret_cast<const float4*>(stg + j * STG_LD + sub * 16);
+          float x[16];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 v = s4[i];
+            x[4 * i] = v.x;
+            x[4 * i + 1] = v.y;
+            x[4 * i + 2] = v.z;
+            x[4 * i + 3] = v.w;
+          }
+          float mx = -INFINITY, sm = 0.f;
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (i < valid) mx = fmaxf(mx, x[i]);
+          if (mx != -INFINITY) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (i < valid) sm += expf(x[i] - mx);
+          }
+          lse_pair<4>(mx, sm);
+          if (sub == 0 && j < nv) a.lse_part[(size_t)m_tile * a.lse_ld + tok0 + j] = make_float2(mx, sm);
+        } else {   // EPI_SWIGLU: rows 0-63 of the tile are gates, 64-127 the matching ups
           const int f = wt & 31, n0 = wt >> 5;   // two adjacent features, every fourth token
           __nv_bfloat16* out = a.out_bf16 + m_tile * 64 + 2 * f;
 #pragma unroll
@@ -308,6 +336,7 @@ cudaError_t launch_bn(EpiKind e, const CUtensorMap& ma, const CUtensorMap& mb, c
     case EPI_F32: return launch_t<BN, EPI_F32>(ma, mb, kp, st);
     case EPI_RESID: return launch_t<BN, EPI_RESID>(ma, mb, kp, st);
     case EPI_SWIGLU: return launch_t<BN, EPI_SWIGLU>(ma, mb, kp, st);
+    case EPI_LSE: return launch_t<BN, EPI_LSE>(ma, mb, kp, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -323,7 +352,7 @@ int cluster_size(long long tiles, int kb, int sms) {
 }  // namespace
 
 bool gemm_cluster_fits(const GemmArgs& a, int sms) {
-  if (a.epi != EPI_F32 && a.epi != EPI_RESID && a.epi != EPI_SWIGLU) return false;
+  if (a.epi != EPI_F32 && a.epi != EPI_RESID && a.epi != EPI_SWIGLU && a.epi != EPI_LSE) return false;
   // One token tile: always (so that up to 256 tokens the k-split does not depend on the token count).
   // More: while the grid cannot give every SM a whole tile.  At the line (us, cluster / stream-K):
   // 172 weight tiles x 120 tokens 37.5 / 39.2 and x 200 tokens 52.0 / 49.5; 96 tiles x 2 token tiles

@@ -368,6 +368,18 @@ __device__ __forceinline__ void ws_reduce_resnorm_half(const GemmArgs& a, const 
 // 32-token chunk)
 __device__ __forceinline__ float swiglu(float g, float u) { return __fdividef(g, 1.0f + __expf(-g)) * u; }
 
+// Combines (max, sum of exp(y - max)) over the lanes that differ in the bits up to MAXO, pairs first.
+template <int MAXO>
+__device__ __forceinline__ void lse_pair(float& mx, float& sm) {
+#pragma unroll
+  for (int o = 1; o <= MAXO; o <<= 1) {
+    const float m2 = __shfl_xor_sync(0xffffffffu, mx, o), s2 = __shfl_xor_sync(0xffffffffu, sm, o);
+    const float mn = fmaxf(mx, m2);
+    sm = (mx == -INFINITY ? 0.f : sm * expf(mx - mn)) + (m2 == -INFINITY ? 0.f : s2 * expf(m2 - mn));
+    mx = mn;
+  }
+}
+
 // st: staging [32 tokens][128 rows] fp32 of one chunk; 128 threads (ep_tid) write the outputs.
 // tpos / tkvr: the n-tile's token tables (EPI_QKV only); trs: the n-tile's norm scales (EPI_QKV /
 // EPI_SWIGLU when the input rows are g * h, else null).
@@ -494,13 +506,7 @@ __device__ __forceinline__ void epi_chunk(const GemmArgs& a, const float* st, in
         if (sub * 32 + r < valid) sm += expf(sj[r] - mx);
       }
     }
-#pragma unroll
-    for (int o = 1; o <= 2; o <<= 1) {
-      const float m2 = __shfl_xor_sync(0xffffffffu, mx, o), s2 = __shfl_xor_sync(0xffffffffu, sm, o);
-      const float mn = fmaxf(mx, m2);
-      sm = (mx == -INFINITY ? 0.f : sm * expf(mx - mn)) + (m2 == -INFINITY ? 0.f : s2 * expf(m2 - mn));
-      mx = mn;
-    }
+    lse_pair<2>(mx, sm);
     const int tok = tok0 + j;
     if (sub == 0 && tok < a.T) a.lse_part[(size_t)m_tile * a.lse_ld + tok] = make_float2(mx, sm);
   } else {

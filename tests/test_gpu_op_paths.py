@@ -125,3 +125,34 @@ def test_attention_paths(ats, H, hd, P, T, paths):
         mag = mag + torch.einsum("htj,tjhd->thd", w[:, :, P:], pv.abs())
     # the weights are rounded to fp16 (2^-11), the result to bf16
     assert bool(((out - ref).abs() <= 2.0 ** -8 * ref.abs() + 2.0 ** -11 * mag + 1e-5).all())
+
+
+# whole-vocabulary log-sum-exp (FULL normalisation): one token tile of every width, several; a partial last
+# weight tile; enough tiles for the CTA pairs (an odd and an even count)
+@pytest.mark.parametrize("V,users,N,gamma", [(1200, 1, 7, 1), (1200, 3, 17, 1), (2000, 2, 40, 1), (1200, 1, 80, 3),
+                                             (1025, 3, 100, 3), (33024, 1, 100, 3), (16500, 4, 100, 3)])
+def test_full_lse_paths(ats, V, users, N, gamma):
+    from types import SimpleNamespace
+    d, f = 64, 128
+    w = {"embed": _randn((V, d), 1), "lm_head": _randn((V, d), 2, 0.4), "final_norm": _randn((d,), 3, 0.1) + 1}
+    for name, shape in (("attn_norm", (d,)), ("mlp_norm", (d,)), ("wqkv", (3 * d, d)), ("wo", (d, d)),
+                        ("wgate_up", (2 * f, d)), ("wdown", (d, f))):
+        w["layers.0." + name] = _randn(shape, 4 + len(name), 0.1)
+    spec = SimpleNamespace(n_layers=1, d_model=d, n_heads=2, d_ffn=f, vocab=V, rms_eps=1e-6, rope_theta=1e4)
+    items = np.zeros((256, 4), np.int32)
+    items[:, 0] = np.arange(256)
+    ctx = ats.Context(spec, w, None, None, items, 0, max_users=users, max_prompt=8, max_K=5, max_N=N, max_gamma=gamma)
+    o = ats.opts(5, N, gamma, norm=ats.NORM_FULL)
+    ctx.prefill(torch.arange(8 * users, dtype=torch.int32, device="cuda"), 8 * np.arange(users + 1))
+    ctx.begin_step(o)
+    parents, codes = np.zeros((2, users, gamma, N), np.int32)
+    parents[:, 1:], codes[:, 0] = np.arange(N), np.arange(N)
+    ctx.set_tree(np.full((users, gamma), N), parents, codes, np.zeros((users, gamma, N)))
+    ctx.verify(o, ats.STRICT)
+    T = users * gamma * N
+    x = torch.from_numpy(ctx.debug_buffer(0, 1, np.int16, T * d).reshape(T, d)).cuda().view(torch.bfloat16)
+    ref = torch.logsumexp(x.double() @ w["lm_head"].double().T, 1)
+    got = torch.from_numpy(ctx.debug_buffer(0, 10, np.float32, users + T)[users:]).cuda().double()
+    # fp32 logits (|x . w| up to ~30) and exponentials of them: a few units of 2^-23 of the largest logit
+    assert float((got - ref).abs().max()) < 2e-5
+    ctx.close()
