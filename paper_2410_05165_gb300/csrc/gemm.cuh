@@ -98,7 +98,6 @@ cudaError_t gemm_cluster_launch(const GemmArgs& a, unsigned int* err, int sms, c
 
 // The GEMM with many tiles and more than one token tile (gemm_pair.cu): EPI_F32, EPI_RESID, EPI_SWIGLU and
 // EPI_LSE on a grid of `grid` CTAs (gemm_grid_size).
-bool gemm_pair_fits(const GemmArgs& a, int grid);
 cudaError_t gemm_pair_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaStream_t stream, char* errbuf,
                              size_t errlen);
 

@@ -3,7 +3,8 @@
 // its N), another decomposition:
 //
 //   * one cluster of C CTAs (C <= 8) per tile of 128 weight rows x BN tokens; CTA r streams the r-th
-//     share of the k-blocks through its TMA ring into its own TMEM accumulator;
+//     share of the k-blocks through its TMA ring into two TMEM accumulators, half of the share each (the
+//     tensor core rounds towards zero, so the error grows with the length of an accumulation);
 //   * the partial sums meet in distributed shared memory: the tile's 16-token groups are dealt out to
 //     the CTAs, every CTA stores its partial of a group straight into the owner's shared memory (the
 //     ring, idle by then), and the owner adds the C partials in CTA order and runs the epilogue.
@@ -14,19 +15,27 @@
 // on the weight shape and the number of token tiles alone, so a token's result does not depend on the
 // other tokens of the call (one token tile up to 256 tokens).
 //
-// Measured against the stream-K kernel (us, GB300): [12288 x 4096] x 120 tokens 32.1 -> 24.4 (4.4 TB/s),
-// [4096 x 11008] x 120 31.4 -> 24.7, [4096 x 4096] x 120 23.3 -> 16.4, [768 x 768] x 10 9.4 -> 6.6,
-// [4096 x 11008] x 512 56.6 -> 45.8, [4096 x 11008] x 960 90.2 -> 72.6.
+// A CTA takes a whole SM (220 KB ring: 7 k-blocks in flight at 128 tokens), one wave.  Only where the
+// tiles alone are more than the SMs (C = 1) do two share one ("narrow": 96 KB ring, one accumulator), so
+// that the second wave's CTAs run beside the first's.  Two per SM and larger clusters were slower where
+// one wave is enough: half the copies in flight per CTA and more partials to exchange.
 //
-// A CTA takes at most half an SM's shared memory (96 KB ring, two CTAs per SM), so up to 304 CTAs
-// stream at once and one CTA's exchange overlaps the other's stream.
-// Bound: HBM up to ~256 tokens (weights once), the tensor pipe and the ring's fill rate above.
+// Measured against the stream-K kernel / two narrow CTAs per SM (us, GB300): [12288 x 4096] x 120 tokens
+// 32.1 / 23.7 -> 22.7 (4.5 TB/s), x 200 31.4 -> 29.4 (narrow), x 10 20.1 -> 21.4 (narrow; the one loss: an SM
+// takes in 60 bytes per ns, and 96 of 152 are used), [4096 x 11008] x 120 31.4 / 24.7 -> 20.6, x 200 35.6
+// -> 25.7 (narrow), [4096 x 4096] x 120 23.3 / 16.2 -> 12.4, [768 x 768] x 10 9.4 / 6.5 -> 5.8, [4096 x 11008] x
+// 512 56.6 / 46.3 -> 40.7, x 960 90.2 / 72.6 -> 67.0.
+// Error against fp64 (relative, stream-K kernel / here): [4096 x 11008] 2.3e-6 / 1.4e-6, [4096 x 4096] 7.9e-7 /
+// 4.7e-7, [768 x 768] 0.9e-7 / 1.1e-7, [22016 x 4096] 4.2e-6 / 4.4e-6.
+//
+// Bound: HBM and the SM's intake up to ~256 tokens (weights once), the tensor pipe and the ring's fill
+// rate above.
 //
 // Roles (320 threads): warp 0 = TMA producer, warp 1 = TMEM + MMA issue, warps 2-9 = two epilogue
 // warpgroups (TMEM lane quadrant = warp % 4), which alternate the groups they own.
 #include <stdio.h>
 
-#include <algorithm>
+#include <atomic>
 
 #include "common.cuh"
 #include "gemm.cuh"
@@ -39,35 +48,55 @@ namespace {
 constexpr int THREADS = 320;
 constexpr int GROUP = 16;                            // tokens of an exchange group
 constexpr int GROUP_FLOATS = GROUP * GEMM_BM;        // one CTA's partial of a group: [token/4][row][4]
-constexpr int ROUND = 128;                           // tokens exchanged at once (bounds the receive area)
 constexpr int STG_LD = GEMM_BM + 4;                  // staging row of one token (SwiGLU), floats
-constexpr int MAX_CLUSTER = 8;
 
 template <int BN>
 struct KCfg {
   static constexpr int A_BYTES = GEMM_BM * 128;
   static constexpr int B_BYTES = BN * 128;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+  // copies in flight: two CTAs per SM, or one ("wide")
   static constexpr int STAGES = BN >= 256 ? 2 : BN >= 128 ? 3 : BN >= 64 ? 4 : 5;
-  static constexpr int RING = STAGES * STAGE_BYTES;
-  // after the last MMA: receive area (a CTA owns at most ceil(8 / C) groups of a round, each with
-  // C - 1 received partials), then a staging buffer per warpgroup
-  static constexpr int RECV_GROUPS = 10;
-  static constexpr int STG_OFF = RECV_GROUPS * GROUP_FLOATS * 4;
+  static constexpr int WIDE_STAGES = (232448 - 1024 - 256) / STAGE_BYTES;
+  // after the last MMA: (wide) receive area, a CTA owns at most ceil(groups / C) groups, each with C - 1
+  // received partials; then a staging buffer per warpgroup
+  static constexpr int RECV_GROUPS = BN >= 256 ? 15 : 10;
   static constexpr int STG_BYTES = 16 * STG_LD * 4;
-  static constexpr int BODY = STG_OFF + 2 * STG_BYTES > RING ? STG_OFF + 2 * STG_BYTES : RING;
-  static constexpr int SMEM = 1024 + BODY + 256;
-  static_assert(SMEM <= 113 * 1024, "two CTAs per SM");
+  static constexpr int stg_off(bool wide) { return wide ? RECV_GROUPS * GROUP_FLOATS * 4 : 0; }
+  static constexpr int body(bool wide) {
+    const int ring = (wide ? WIDE_STAGES : STAGES) * STAGE_BYTES, exch = stg_off(wide) + 2 * STG_BYTES;
+    return ring > exch ? ring : exch;
+  }
+  static constexpr int smem(bool wide) { return 1024 + body(wide) + 256; }
+  static_assert(smem(false) <= 113 * 1024, "two CTAs per SM");
+  static_assert(smem(true) <= 232448 && smem(true) > 117 * 1024, "one CTA per SM");
 };
 
 struct KcParams {
   GemmArgs a;
   int m_tiles, n_tiles, kb, C, up_row0;
+  bool wide;
   unsigned int* err;
 };
 
-__device__ __forceinline__ void st_cluster_f4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+__device__ __forceinline__ void st_cluster_f4(uint32_t addr, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
+// A CTA's partial of 16 tokens of its TMEM lane's row: the sum of its accumulators (the second's
+// `second` columns on, 0: none).
+__device__ __forceinline__ void ld_group(uint32_t addr, uint32_t second, float (&v)[16]) {
+  uint32_t r[16];
+  tmem_ld_32x32b_x16(addr, r);
+  tmem_ld_wait();
+#pragma unroll
+  for (int n = 0; n < 16; ++n) v[n] = __uint_as_float(r[n]);
+  if (second) {
+    tmem_ld_32x32b_x16(addr + second, r);
+    tmem_ld_wait();
+#pragma unroll
+    for (int n = 0; n < 16; ++n) v[n] += __uint_as_float(r[n]);
+  }
 }
 
 template <int BN, int EPI>
@@ -77,9 +106,10 @@ __global__ void __launch_bounds__(THREADS, 2)
   using C = KCfg<BN>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::BODY);
-  uint64_t* empty = full + C::STAGES;
-  uint64_t* tfull = empty + C::STAGES;
+  const int stages = p.wide ? C::WIDE_STAGES : C::STAGES;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::body(p.wide));
+  uint64_t* empty = full + stages;
+  uint64_t* tfull = empty + stages;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull + 1);
   int* failed = reinterpret_cast<int*>(tmem_slot + 1);
 
@@ -88,9 +118,10 @@ __global__ void __launch_bounds__(THREADS, 2)
   const int tile = blockIdx.x / nc;
   const int m_tile = tile / p.n_tiles, n_tile = tile % p.n_tiles;
   const int k0 = rank * p.kb / nc, k1 = (rank + 1) * p.kb / nc;   // this CTA's k-blocks (never empty: C <= kb)
+  const int k2 = p.wide ? k0 + (k1 - k0 + 1) / 2 : k1;             // the second accumulator's first
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < C::STAGES; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -99,7 +130,7 @@ __global__ void __launch_bounds__(THREADS, 2)
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, BN);
+    tmem_alloc(tmem_slot, (uint32_t)(p.wide ? 2 * BN : BN));
     tmem_relinquish();
   }
   tc_fence_before();
@@ -133,7 +164,7 @@ __global__ void __launch_bounds__(THREADS, 2)
         tma_load_2d(sa, &tmA, &full[stage], k * GEMM_BK, r0, pol_w);
         tma_load_2d(sa + 8192, &tmA, &full[stage], k * GEMM_BK, r1, pol_w);
         tma_load_2d(sa + C::A_BYTES, &tmB, &full[stage], k * GEMM_BK, n_tile * BN, pol_x);
-        if (++stage == C::STAGES) {
+        if (++stage == stages) {
           stage = 0;
           phase ^= 1u;
         }
@@ -155,9 +186,10 @@ __global__ void __launch_bounds__(THREADS, 2)
         const uint64_t ad = smem_desc_sw128(sa), bd = smem_desc_sw128(sa + C::A_BYTES);
 #pragma unroll
         for (int kk = 0; kk < GEMM_BK / 16; ++kk)
-          tc_mma_bf16(tmem_base, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc, (k > k0 || kk > 0) ? 1u : 0u);
+          tc_mma_bf16(k < k2 ? tmem_base : tmem_base + BN, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc,
+                      ((k != k0 && k != k2) || kk > 0) ? 1u : 0u);
         tc_commit(&empty[stage]);
-        if (++stage == C::STAGES) {
+        if (++stage == stages) {
           stage = 0;
           phase ^= 1u;
         }
@@ -182,143 +214,136 @@ __global__ void __launch_bounds__(THREADS, 2)
   const int m = (warp & 3) * 32 + lane;                               // TMEM lane = row of the tile
   const uint32_t tb = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
   float* recv = reinterpret_cast<float*>(smem);
-  float* stg = reinterpret_cast<float*>(smem + C::STG_OFF + (wg & 1) * C::STG_BYTES);
+  float* stg = reinterpret_cast<float*>(smem + C::stg_off(p.wide) + (wg & 1) * C::STG_BYTES);
   const int nvalid = min(BN, a.T - n_tile * BN);
+  const uint32_t second = k2 < k1 ? BN : 0;   // the second accumulator's columns
   if (nc > 1) cluster_sync();   // every CTA's ring is idle: it may receive partials
-#pragma unroll 1
-  for (int t0 = 0; t0 < nvalid; t0 += ROUND) {
-    const int ng = (min(ROUND, nvalid - t0) + GROUP - 1) / GROUP;   // groups of this round: owner = group % C
-    if (nc > 1) {
-      if (warp >= 2) {
-#pragma unroll 1
-        for (int g = wg; g < ng; g += 2) {
-          const int owner = g % nc;
-          if (owner == rank) continue;
-          uint32_t r[16];
-          tmem_ld_32x32b_x16(tb + t0 + g * GROUP, r);
-          tmem_ld_wait();
-          // slot of (group, source) in the owner's receive area
-          const int slot = (g / nc) * (nc - 1) + (rank < owner ? rank : rank - 1);
-          const uint32_t dst = mapa_u32(recv + slot * GROUP_FLOATS + m * 4, (uint32_t)owner);
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            st_cluster_f4(dst + j * (GEMM_BM * 16), r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
-        }
-      }
-      cluster_sync();   // the partials of every group are in place
-    }
+  const int ng = (nvalid + GROUP - 1) / GROUP;   // groups: owner = group % C
+  if (nc > 1) {
     if (warp >= 2) {
 #pragma unroll 1
-      for (int g = rank + wg * nc; g < ng; g += 2 * nc) {
-        const int tok0 = n_tile * BN + t0 + g * GROUP, nv = min(GROUP, a.T - tok0);
-        const int row = m_tile * GEMM_BM + m;
-        float old[16];
-        if constexpr (EPI == EPI_RESID) {
+      for (int g = wg; g < ng; g += 2) {
+        const int owner = g % nc;
+        if (owner == rank) continue;
+        float r[16];
+        ld_group(tb + g * GROUP, second, r);
+        // slot of (group, source) in the owner's receive area
+        const int slot = (g / nc) * (nc - 1) + (rank < owner ? rank : rank - 1);
+        const uint32_t dst = mapa_u32(recv + slot * GROUP_FLOATS + m * 4, (uint32_t)owner);
 #pragma unroll
-          for (int n = 0; n < GROUP; ++n)
-            old[n] = row < a.M && n < nv ? __ldcg(a.out_f32 + (size_t)(tok0 + n) * a.ldo + row) : 0.f;
-        }
-        uint32_t own[16];
-        tmem_ld_32x32b_x16(tb + t0 + g * GROUP, own);
-        tmem_ld_wait();
-        float acc[16];
-#pragma unroll
-        for (int n = 0; n < GROUP; ++n) acc[n] = rank == 0 ? __uint_as_float(own[n]) : 0.f;
+        for (int j = 0; j < 4; ++j)
+          st_cluster_f4(dst + j * (GEMM_BM * 16), make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]));
+      }
+    }
+    cluster_sync();   // the partials of every group are in place
+  }
+  if (warp >= 2) {
 #pragma unroll 1
-        for (int src = 0; src < nc; ++src) {   // CTA order
-          if (src == rank) {
-            if (rank > 0) {
+    for (int g = rank + wg * nc; g < ng; g += 2 * nc) {
+      const int tok0 = n_tile * BN + g * GROUP, nv = min(GROUP, a.T - tok0);
+      const int row = m_tile * GEMM_BM + m;
+      float old[16];
+      if constexpr (EPI == EPI_RESID) {
 #pragma unroll
-              for (int n = 0; n < GROUP; ++n) acc[n] += __uint_as_float(own[n]);
-            }
-            continue;
-          }
-          const int slot = (g / nc) * (nc - 1) + (src < rank ? src : src - 1);
-          const float4* q = reinterpret_cast<const float4*>(recv + slot * GROUP_FLOATS) + m;
+        for (int n = 0; n < GROUP; ++n)
+          old[n] = row < a.M && n < nv ? __ldcg(a.out_f32 + (size_t)(tok0 + n) * a.ldo + row) : 0.f;
+      }
+      float own[16], acc[16];
+      ld_group(tb + g * GROUP, second, own);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float4 v = q[j * GEMM_BM];
-            acc[4 * j] += v.x;
-            acc[4 * j + 1] += v.y;
-            acc[4 * j + 2] += v.z;
-            acc[4 * j + 3] += v.w;
-          }
-        }
-        if constexpr (EPI == EPI_F32 || EPI == EPI_RESID) {
-          if (row < a.M) {
-            float* o = a.out_f32 + (size_t)tok0 * a.ldo + row;
+      for (int n = 0; n < GROUP; ++n) acc[n] = rank == 0 ? own[n] : 0.f;
+#pragma unroll 1
+      for (int src = 0; src < nc; ++src) {   // CTA order
+        if (src == rank) {
+          if (rank > 0) {
 #pragma unroll
-            for (int n = 0; n < GROUP; ++n)
-              if (n < nv) o[(size_t)n * a.ldo] = EPI == EPI_RESID ? old[n] + acc[n] : acc[n];
+            for (int n = 0; n < GROUP; ++n) acc[n] += own[n];
           }
           continue;
         }
-        named_bar_sync(1 + wg, 128);   // the previous group's rows have been read
+        const int slot = (g / nc) * (nc - 1) + (src < rank ? src : src - 1);
+        const float4* q = reinterpret_cast<const float4*>(recv + slot * GROUP_FLOATS) + m;
 #pragma unroll
-        for (int n = 0; n < GROUP; ++n) stg[n * STG_LD + m] = acc[n];
-        named_bar_sync(1 + wg, 128);
-        if constexpr (EPI == EPI_LSE) {
-          // (max, sum of exp(y - max)) of each token over the tile's rows: eight threads per token, 16 rows
-          // each (four at a time), then combined in a fixed order
-          const int j = wt >> 3, sub = wt & 7;
-          const int valid = min(GEMM_BM, a.M - m_tile * GEMM_BM) - sub * 16;
-          const float4* s4 = reinterpret_cast<const float4*>(stg + j * STG_LD + sub * 16);
-          float x[16];
+        for (int j = 0; j < 4; ++j) {
+          const float4 v = q[j * GEMM_BM];
+          acc[4 * j] += v.x;
+          acc[4 * j + 1] += v.y;
+          acc[4 * j + 2] += v.z;
+          acc[4 * j + 3] += v.w;
+        }
+      }
+      if constexpr (EPI == EPI_F32 || EPI == EPI_RESID) {
+        if (row < a.M) {
+          float* o = a.out_f32 + (size_t)tok0 * a.ldo + row;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float4 v = s4[i];
-            x[4 * i] = v.x;
-            x[4 * i + 1] = v.y;
-            x[4 * i + 2] = v.z;
-            x[4 * i + 3] = v.w;
-          }
-          float mx = -INFINITY, sm = 0.f;
+          for (int n = 0; n < GROUP; ++n)
+            if (n < nv) o[(size_t)n * a.ldo] = EPI == EPI_RESID ? old[n] + acc[n] : acc[n];
+        }
+        continue;
+      }
+      named_bar_sync(1 + wg, 128);   // the previous group's rows have been read
+#pragma unroll
+      for (int n = 0; n < GROUP; ++n) stg[n * STG_LD + m] = acc[n];
+      named_bar_sync(1 + wg, 128);
+      if constexpr (EPI == EPI_LSE) {
+        // (max, sum of exp(y - max)) of each token over the tile's rows: eight threads per token, 16 rows
+        // each (four at a time), then combined in a fixed order
+        const int j = wt >> 3, sub = wt & 7;
+        const int valid = min(GEMM_BM, a.M - m_tile * GEMM_BM) - sub * 16;
+        const float4* s4 = reinterpret_cast<const float4*>(stg + j * STG_LD + sub * 16);
+        float x[16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float4 v = s4[i];
+          x[4 * i] = v.x;
+          x[4 * i + 1] = v.y;
+          x[4 * i + 2] = v.z;
+          x[4 * i + 3] = v.w;
+        }
+        float mx = -INFINITY, sm = 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (i < valid) mx = fmaxf(mx, x[i]);
+        if (mx != -INFINITY) {
 #pragma unroll
           for (int i = 0; i < 16; ++i)
-            if (i < valid) mx = fmaxf(mx, x[i]);
-          if (mx != -INFINITY) {
+            if (i < valid) sm += expf(x[i] - mx);
+        }
+        lse_pair<4>(mx, sm);
+        if (sub == 0 && j < nv) a.lse_part[(size_t)m_tile * a.lse_ld + tok0 + j] = make_float2(mx, sm);
+      } else {   // EPI_SWIGLU: rows 0-63 of the tile are gates, 64-127 the matching ups
+        const int f = wt & 31, n0 = wt >> 5;   // two adjacent features, every fourth token
+        __nv_bfloat16* out = a.out_bf16 + m_tile * 64 + 2 * f;
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-              if (i < valid) sm += expf(x[i] - mx);
-          }
-          lse_pair<4>(mx, sm);
-          if (sub == 0 && j < nv) a.lse_part[(size_t)m_tile * a.lse_ld + tok0 + j] = make_float2(mx, sm);
-        } else {   // EPI_SWIGLU: rows 0-63 of the tile are gates, 64-127 the matching ups
-          const int f = wt & 31, n0 = wt >> 5;   // two adjacent features, every fourth token
-          __nv_bfloat16* out = a.out_bf16 + m_tile * 64 + 2 * f;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int n = n0 + 4 * k;
-            if (n < nv) {
-              const float2 gv = *reinterpret_cast<const float2*>(stg + n * STG_LD + 2 * f);
-              const float2 uv = *reinterpret_cast<const float2*>(stg + n * STG_LD + 64 + 2 * f);
-              *reinterpret_cast<__nv_bfloat162*>(out + (size_t)(tok0 + n) * a.ldo) =
-                  __floats2bfloat162_rn(swiglu(gv.x, uv.x), swiglu(gv.y, uv.y));
-            }
+        for (int k = 0; k < 4; ++k) {
+          const int n = n0 + 4 * k;
+          if (n < nv) {
+            const float2 gv = *reinterpret_cast<const float2*>(stg + n * STG_LD + 2 * f);
+            const float2 uv = *reinterpret_cast<const float2*>(stg + n * STG_LD + 64 + 2 * f);
+            *reinterpret_cast<__nv_bfloat162*>(out + (size_t)(tok0 + n) * a.ldo) =
+                __floats2bfloat162_rn(swiglu(gv.x, uv.x), swiglu(gv.y, uv.y));
           }
         }
       }
     }
-    // (a further round overwrites the receive areas that this one reads)
-    if (nc > 1 && t0 + ROUND < nvalid) cluster_sync();
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, BN);
+    tmem_dealloc(tmem_base, (uint32_t)(p.wide ? 2 * BN : BN));
   }
 }
 
 template <int BN, int EPI>
 cudaError_t launch_t(const CUtensorMap& ma, const CUtensorMap& mb, const KcParams& kp, cudaStream_t st) {
   static std::atomic<unsigned long long> attr_done{0};
-  const cudaError_t e = smem_attr_once(attr_done, gemm_cluster_kernel<BN, EPI>, KCfg<BN>::SMEM);
+  const cudaError_t e = smem_attr_once(attr_done, gemm_cluster_kernel<BN, EPI>, KCfg<BN>::smem(true));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(kp.m_tiles * kp.n_tiles * kp.C));
   cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = KCfg<BN>::SMEM;
+  cfg.dynamicSmemBytes = KCfg<BN>::smem(kp.wide);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -341,12 +366,18 @@ cudaError_t launch_bn(EpiKind e, const CUtensorMap& ma, const CUtensorMap& mb, c
   }
 }
 
-// CTAs of a tile's cluster: as many as keep every CTA of the grid resident at once (two per SM), one
-// k-block at least each.  (Not 7: its receive area would not fit.)
+// CTAs of a tile's cluster: as many as can all run at once, one per SM, with three k-blocks each at
+// least.  On 152 SMs there is room for 76 clusters of two, 46 of three, 36 of four, 23 of six, 15 of eight;
+// a cluster that has to wait costs a second wave (us, 120 tokens, C = 3 / 4 / 6 / 8: 24 weight tiles x 64
+// k-blocks 13.1 / 11.6 / 20.4 / 15.2, 19 x 64 13.0 / 11.4 / 11.4 / 20.1), and eight are better than six only
+// where six would leave most SMs idle (12 x 64: 10.5 with six, 11.0 with eight; 2 x 172, 10 tokens: 13.6,
+// 12.3).  Small K: 6 x 12, C = 2 / 3 / 4 / 6 / 8: 6.1 / 6.2 / 6.1 / 6.4 / 6.9.
 int cluster_size(long long tiles, int kb, int sms) {
-  long long c = std::max<long long>(1, 2LL * sms / tiles);
-  c = std::min<long long>(c, std::min(kb, MAX_CLUSTER));
-  return c == 7 ? 6 : (int)c;
+  auto fits = [&](int c, int room) { return tiles * c <= room && kb >= 3 * c; };
+  if (fits(8, sms / 2)) return 8;
+  for (int c : {6, 4, 3})
+    if (fits(c, sms * 9 / 10)) return c;
+  return fits(2, sms) ? 2 : 1;
 }
 
 }  // namespace
@@ -354,9 +385,8 @@ int cluster_size(long long tiles, int kb, int sms) {
 bool gemm_cluster_fits(const GemmArgs& a, int sms) {
   if (a.epi != EPI_F32 && a.epi != EPI_RESID && a.epi != EPI_SWIGLU && a.epi != EPI_LSE) return false;
   // One token tile: always (so that up to 256 tokens the k-split does not depend on the token count).
-  // More: while the grid cannot give every SM a whole tile.  At the line (us, cluster / stream-K):
-  // 172 weight tiles x 120 tokens 37.5 / 39.2 and x 200 tokens 52.0 / 49.5; 96 tiles x 2 token tiles
-  // (192 in all) 51.4 / 50.9, 32 x 4 (128) 72.6 / 90.2.
+  // More: while every tile has an SM of its own.  At the line (us, cluster / CTA pairs, K = 4096): 128 tiles
+  // ([8192] x 512 tokens) 29.7 / 41.2, 160 ([5120] x 1000) 47.5 / 51.6, 192 ([12288] x 512) 56.5 / 41.9.
   if (a.T <= 256) return true;
   const long long m_tiles = a.epi == EPI_SWIGLU ? a.M / 128 : ((long long)a.M + 127) / 128;
   return m_tiles * ((a.T + 255) / 256) <= sms;
@@ -374,6 +404,7 @@ cudaError_t gemm_cluster_launch(const GemmArgs& a, unsigned int* err, int sms, c
   kp.up_row0 = a.epi == EPI_SWIGLU ? a.M / 2 : 0;
   kp.kb = a.K / GEMM_BK;
   kp.C = cluster_size((long long)kp.m_tiles * kp.n_tiles, kp.kb, sms);
+  kp.wide = (long long)kp.m_tiles * kp.n_tiles <= sms;
   kp.err = err;
   CUtensorMap ma, mb;
   if (!gemm_make_map(&ma, a.W, a.K, a.M, 64, eb, el)) return kGemmMapError;

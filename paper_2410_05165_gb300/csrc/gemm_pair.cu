@@ -291,14 +291,6 @@ cudaError_t launch_t(const CUtensorMap& ma, const CUtensorMap& mb, const PairPar
 
 }  // namespace
 
-bool gemm_pair_fits(const GemmArgs& a, int grid) {
-  if (a.epi != EPI_F32 && a.epi != EPI_RESID && a.epi != EPI_SWIGLU && a.epi != EPI_LSE) return false;
-  const long long m_tiles = a.epi == EPI_SWIGLU ? a.M / 128 : ((long long)a.M + 127) / 128;
-  // More than one token tile (a single one is bound by the weights' stream), and a whole tile for every
-  // pair.
-  return a.T > 256 && (m_tiles + 1) / 2 * ((a.T + BN - 1) / BN) >= grid / 2;
-}
-
 cudaError_t gemm_pair_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaStream_t stream, char* eb,
                              size_t el) {
   const cudaError_t ce = gemm_check(a, s.max_tiles, eb, el);

@@ -33,7 +33,7 @@ def _x(T, K, seed):
 GEMM = [(1, 64, 1), (127, 64, 16), (129, 128, 17), (300, 192, 31), (128, 448, 32), (640, 512, 33), (2304, 768, 64),
         (1920, 1024, 65), (1000, 2048, 127), (4096, 1024, 128), (768, 4096, 129), (3000, 640, 250), (6400, 256, 256),
         (256, 1024, 257), (900, 512, 300), (4096, 640, 512), (12900, 320, 100), (20000, 256, 200), (22016, 128, 130),
-        (4096, 320, 900)]
+        (4096, 320, 900), (2000, 1600, 40), (2304, 1344, 70), (3900, 11008, 60)]
 
 
 @pytest.mark.parametrize("M,K,T", GEMM)
