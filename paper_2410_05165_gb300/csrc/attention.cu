@@ -4,6 +4,7 @@
 #include <cudaTypedefs.h>
 #include <math.h>
 #include <stdio.h>
+#include <string.h>
 
 #include "attention.cuh"
 #include "attn_core.cuh"
@@ -94,10 +95,18 @@ struct AttClusterSink {
   }
 };
 
-template <int HD>
+// The call's tables in the kernel's parameters (NTAB ints), or in memory (NTAB = 0).
+template <int NTAB>
+struct AttTables {
+  int v[NTAB > 0 ? NTAB : 1];
+};
+
+template <int HD, int NTAB>
 __global__ void __launch_bounds__(128, 3)
-    attn_cluster_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv, const AttnArgs a,
-                        const int S) {
+    attn_cluster_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv,
+                        const AttnArgs args, const int S, const int paths, const __grid_constant__ AttTables<NTAB> tab) {
+  AttnArgs a = args;
+  if constexpr (NTAB > 0) attn_tables(a, tab.v, paths);
   using CC = AttClusterCfg<HD>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -204,12 +213,21 @@ __global__ void __launch_bounds__(128, 3)
   }
 }
 
-template <int HD>
-cudaError_t launch_cluster(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, int S, cudaStream_t st) {
+template <int HD, int NTAB>
+cudaError_t launch_cluster(AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, int S, const int* tables,
+                           size_t n, bool paths, int* d_tables, cudaStream_t st) {
   using CC = AttClusterCfg<HD>;
   static std::atomic<unsigned long long> attr_done{0};
-  const cudaError_t e = smem_attr_once(attr_done, attn_cluster_kernel<HD>, CC::SMEM);
+  cudaError_t e = smem_attr_once(attr_done, attn_cluster_kernel<HD, NTAB>, CC::SMEM);
   if (e != cudaSuccess) return e;
+  AttTables<NTAB> tab;
+  if constexpr (NTAB > 0) {
+    memcpy(tab.v, tables, n * sizeof(int));
+  } else {
+    e = cudaMemcpyAsync(d_tables, tables, n * sizeof(int), cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
+    attn_tables(a, d_tables, paths);
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.n_qtiles * a.n_heads * S));
   cfg.blockDim = dim3(128);
@@ -222,7 +240,20 @@ cudaError_t launch_cluster(const AttnArgs& a, const CUtensorMap& mk, const CUten
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = S > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, attn_cluster_kernel<HD>, mk, mv, a, S);
+  int with_paths = paths;
+  void* kargs[] = {const_cast<CUtensorMap*>(&mk), const_cast<CUtensorMap*>(&mv), &a, &S, &with_paths, &tab};
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(attn_cluster_kernel<HD, NTAB>), kargs);
+}
+
+template <int HD>
+cudaError_t launch_cluster_hd(AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, int S, const int* tables,
+                              size_t n, bool paths, int* d_tables, cudaStream_t st) {
+  // Tables as kernel parameters (32,764 bytes at most): no copy ahead of the kernel.  Two sizes, since the
+  // whole parameter block is copied at the launch.  120 tree tokens of 32 heads (740 ints), us per call:
+  // through memory 39, 7680 ints 38, 1984 ints 34-36; 1000 prefill tokens (1081 ints): 44 -> 39.
+  if (n <= 1984) return launch_cluster<HD, 1984>(a, mk, mv, S, tables, n, paths, d_tables, st);
+  if (n <= 7680) return launch_cluster<HD, 7680>(a, mk, mv, S, tables, n, paths, d_tables, st);
+  return launch_cluster<HD, 0>(a, mk, mv, S, tables, n, paths, d_tables, st);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn_att() {
@@ -304,11 +335,12 @@ cudaError_t attn_launch(const AttnArgs& a, const CUtensorMap& mk, const CUtensor
   return cudaErrorInvalidValue;
 }
 
-cudaError_t attn_cluster_launch(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, int S, cudaStream_t st) {
+cudaError_t attn_cluster_launch(AttnArgs a, const CUtensorMap& mk, const CUtensorMap& mv, int S, const int* tables,
+                                size_t n, bool paths, int* d_tables, cudaStream_t st) {
   switch (a.head_dim) {
-    case 32: return launch_cluster<32>(a, mk, mv, S, st);
-    case 64: return launch_cluster<64>(a, mk, mv, S, st);
-    case 128: return launch_cluster<128>(a, mk, mv, S, st);
+    case 32: return launch_cluster_hd<32>(a, mk, mv, S, tables, n, paths, d_tables, st);
+    case 64: return launch_cluster_hd<64>(a, mk, mv, S, tables, n, paths, d_tables, st);
+    case 128: return launch_cluster_hd<128>(a, mk, mv, S, tables, n, paths, d_tables, st);
   }
   return cudaErrorInvalidValue;
 }

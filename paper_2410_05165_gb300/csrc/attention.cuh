@@ -55,8 +55,25 @@ bool attn_make_maps(const __nv_bfloat16* k_cache, const __half* v_cache, int row
 
 cudaError_t attn_launch(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t st, bool pdl);
 
+// The tables of one user's call as one block of ints, at `base`; returns its length.
+__host__ __device__ inline size_t attn_tables(AttnArgs& a, const int* base, bool paths) {
+  a.qt_t0 = base;
+  a.qt_n = a.qt_t0 + a.n_qtiles;
+  a.qt_user = a.qt_n + a.n_qtiles;
+  a.qt_vis = a.qt_user + a.n_qtiles;
+  a.user_splits = a.qt_vis + a.n_qtiles;
+  a.page_table = a.user_splits + 1;
+  a.tok_vis = a.page_table + a.max_pages;
+  a.anc_n = paths ? a.tok_vis + a.T : nullptr;
+  a.anc_row = paths ? a.anc_n + a.T : nullptr;
+  return (size_t)4 * a.n_qtiles + 1 + a.max_pages + (size_t)a.T * (paths ? 6 : 1);
+}
+
 // The same for one user in one kernel: the tile's visible pages over a cluster of S CTAs (1, 2 or 4; the
-// user's user_splits entry), no partials in global memory.  a.direct: S = 1 and no path keys.
-cudaError_t attn_cluster_launch(const AttnArgs& a, const CUtensorMap& mk, const CUtensorMap& mv, int S, cudaStream_t st);
+// user's user_splits entry), no partials in global memory.  a.direct: S = 1 and no path keys.  The tables
+// (attn_tables) are n ints of host memory: they travel as kernel parameters, or, if they are more than
+// those hold, through `d_tables`.
+cudaError_t attn_cluster_launch(AttnArgs a, const CUtensorMap& mk, const CUtensorMap& mv, int S, const int* tables,
+                                size_t n, bool paths, int* d_tables, cudaStream_t st);
 
 }  // namespace atspeed

@@ -166,38 +166,12 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
   for (int t = 0; t < T; ++t) {
     if (h_vis[t] < 0 || h_vis[t] > P) return ATSPEED_E_ARG;
     const int np = h_n_path ? h_n_path[t] : 0;
-    if (np < 0 || np > ATT_MAX_ANC) return ATSPEED_E_ARG;
+    if (np < 0 || np > ATT_MAX_ANC || (np > 0 && !h_path_rows)) return ATSPEED_E_ARG;
     for (int j = 0; j < np; ++j)
       if (h_path_rows[t * 4 + j] < 0 || h_path_rows[t * 4 + j] >= cache_rows) return ATSPEED_E_ARG;
   }
-  int* ip = static_cast<int*>(d_part);
-  std::vector<int> host(4 * nqt + 7 * T + pages + 1, 0);
-  int* qt0 = host.data();
-  int* qtn = qt0 + nqt;
-  int* qtu = qtn + nqt;
-  int* tu = qtu + nqt;
-  int* tv = tu + T;
-  int* an = tv + T;
-  int* ann = an + 4 * T;
-  int* pg = ann + T;
-  int* sp = pg + pages;
-  int* qtv = sp + 1;
-  for (int i = 0; i < nqt; ++i) {
-    qt0[i] = i * ATT_QTILE;
-    qtn[i] = std::min(ATT_QTILE, T - i * ATT_QTILE);
-    qtu[i] = 0;
-  }
-  bool any_path = false;
-  for (int t = 0; t < T; ++t) {
-    any_path |= h_n_path && h_n_path[t] > 0;
-    tv[t] = h_vis[t];
-    qtv[t / ATT_QTILE] = std::max(qtv[t / ATT_QTILE], h_vis[t]);
-    ann[t] = h_n_path ? h_n_path[t] : 0;
-    for (int j = 0; j < 4; ++j) an[t * 4 + j] = (h_path_rows && j < ann[t]) ? h_path_rows[t * 4 + j] : 0;
-  }
-  for (int p = 0; p < pages; ++p) pg[p] = h_pages[p];
-  sp[0] = S;
-  if (cudaMemcpyAsync(ip, host.data(), host.size() * 4, cudaMemcpyHostToDevice, st) != cudaSuccess) return ATSPEED_E_CUDA;
+  bool paths = false;
+  for (int t = 0; h_n_path && t < T; ++t) paths |= h_n_path[t] > 0;
   const int d = n_heads * head_dim;
   CUtensorMap mk, mv;
   char eb[256];
@@ -213,25 +187,31 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
   a.v_cache = static_cast<const __half*>(d_vcache);
   a.kv_rows = cache_rows;
   a.n_qtiles = nqt;
-  const int off_qt0 = 0, off_qtn = nqt, off_qtu = 2 * nqt, off_tu = 3 * nqt, off_tv = off_tu + T, off_an = off_tv + T,
-            off_ann = off_an + 4 * T, off_pg = off_ann + T, off_sp = off_pg + pages, off_qtv = off_sp + 1;
-  a.qt_t0 = ip + off_qt0;
-  a.qt_n = ip + off_qtn;
-  a.qt_user = ip + off_qtu;
-  a.qt_vis = ip + off_qtv;
-  a.tok_user = ip + off_tu;
-  a.tok_vis = ip + off_tv;
-  a.anc_row = ip + off_an;
-  a.anc_n = ip + off_ann;
-  a.page_table = ip + off_pg;
   a.max_pages = std::max(1, pages);
-  a.user_splits = ip + off_sp;
   a.chunks_per_split = 0;
   a.max_splits = S;
   a.out = static_cast<__nv_bfloat16*>(d_out);
-  a.direct = S == 1 && !any_path;
+  a.direct = S == 1 && !paths;
   a.err = nullptr;
-  const cudaError_t e = attn_cluster_launch(a, mk, mv, S, st);
+  std::vector<int> host(attn_tables(a, nullptr, paths), 0);
+  AttnArgs at = a;
+  attn_tables(at, host.data(), paths);
+  auto put = [](const int* p) { return const_cast<int*>(p); };
+  for (int i = 0; i < nqt; ++i) {
+    put(at.qt_t0)[i] = i * ATT_QTILE;
+    put(at.qt_n)[i] = std::min(ATT_QTILE, T - i * ATT_QTILE);
+  }
+  *put(at.user_splits) = S;
+  for (int p = 0; p < pages; ++p) put(at.page_table)[p] = h_pages[p];
+  for (int t = 0; t < T; ++t) {
+    put(at.tok_vis)[t] = h_vis[t];
+    put(at.qt_vis)[t / ATT_QTILE] = std::max(put(at.qt_vis)[t / ATT_QTILE], h_vis[t]);
+    if (!paths) continue;
+    const int na = h_n_path[t];
+    put(at.anc_n)[t] = na;
+    for (int j = 0; j < na; ++j) put(at.anc_row)[t * 4 + j] = h_path_rows[t * 4 + j];
+  }
+  const cudaError_t e = attn_cluster_launch(a, mk, mv, S, host.data(), host.size(), paths, static_cast<int*>(d_part), st);
   return e == cudaSuccess ? ATSPEED_OK : ATSPEED_E_CUDA;
 }
 

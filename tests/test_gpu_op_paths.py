@@ -91,11 +91,12 @@ def test_rmsnorm_paths(ats, T, d, pad):
 
 
 # clusters of 4 (few tiles), 2 and 1 (enough tiles and heads), fewer pages than CTAs, no history at all, queries
-# that see part of it, with and without path keys (one kernel writes its rows directly)
+# that see part of it, with and without path keys (one kernel writes its rows directly), tables of each size
 @pytest.mark.parametrize("H,hd,P,T,paths", [(4, 32, 256, 1, True), (2, 64, 1000, 130, True), (3, 128, 64, 17, True),
                                             (5, 64, 128, 63, False), (32, 128, 200, 330, True), (40, 32, 300, 250, True),
                                             (32, 64, 130, 650, True), (32, 128, 321, 641, False), (2, 32, 0, 5, True),
-                                            (1, 128, 2100, 64, True), (80, 32, 70, 257, False)])
+                                            (1, 128, 2100, 64, True), (80, 32, 70, 257, False), (2, 32, 70, 1300, True),
+                                            (3, 64, 200, 7700, False)])
 def test_attention_paths(ats, H, hd, P, T, paths):
     rng = np.random.default_rng(H + P + T)
     d, n = H * hd, (P + 63) // 64
