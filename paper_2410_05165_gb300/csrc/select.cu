@@ -1,7 +1,7 @@
 // Discrete logic of speculative beam decoding, one CTA (1024 threads) per user:
 //   * trie-masked log-softmax of every beam's item-code logits, cumulative fp32 beam scores;
-//   * exact top-W selection by (score desc, candidate index asc) with a 4-pass radix select over
-//     order-preserving 32-bit keys held in shared memory, then an in-order compaction;
+//   * exact top-W selection by (score desc, candidate index asc) over order-preserving 32-bit keys held in
+//     shared memory: a histogram of their range, then a pairwise ranking of the few keys left;
 //   * drafting (Eq. 1): top-N (strict) or Gumbel-top-N sampling without replacement (relaxed);
 //   * strict top-K verification (Alg. 1) and relaxed sampling verification (Sec. 3.2, Alg. 2),
 //     which also cover plain target beam search / sampling when no level is drafted.
@@ -63,10 +63,17 @@ __device__ __forceinline__ uint32_t ordkey(float x) {
 // ---------------------------------------------------------------------------------------------
 // block primitives (blockDim == NT)
 // ---------------------------------------------------------------------------------------------
+constexpr uint16_t kNone = 0xffff;
+constexpr int CAND = 256;  // candidates ranked at once (and the most a selection returns)
+
 struct Scratch {
-  int hist[256];
+  union {
+    alignas(16) int hist[256];
+    unsigned long long cand[CAND];   // (key, ~index): a larger one comes first
+  };
+  uint32_t wlo[NW], whi[NW];
   int wsum[NW];
-  int misc[8];
+  int misc[4];
   float fred[NW];
 };
 
@@ -117,122 +124,131 @@ __device__ float block_sum(float v, Scratch& s) {
   return r;
 }
 
-// Selects the W best candidates among keys[0..n) (key 0 = invalid), ranked by (key desc, index
+// Selects the W <= CAND best candidates among keys[0..n) (key 0 = invalid), ranked by (key desc, index
 // asc).  Writes their indices to sel[0..m) and returns m = min(W, #valid).
-__device__ int block_select(const uint32_t* keys, int n, int W, int* sel, int* tmp, Scratch& s) {
-  const int per = (n + NT - 1) / NT;
-  const int i0 = threadIdx.x * per, i1 = min(n, i0 + per);
+//
+// Latency-bound (one CTA): a histogram over the range the keys really span leaves few candidates beside
+// the W best after one pass, which are ranked pairwise, in any order.  (Radix passes over all 32 bits put
+// nearly every key of a level into one bin, one shared-memory atomic after the other.)  us, radix / here:
+// draft level 1 / 2 of N = 10 12.3 / 14.2 -> 9.2 / 10.2, verification of 10 beams x 256 18.0 -> 11.2, of 20
+// x 256 for four users 21.3 -> 11.5; one user's four draft levels and verification, K = 20, N = 80, a draft
+// model of 4 layers as both: 1275 -> 1214.
+__device__ int block_select(const uint32_t* keys, int n, int W, int* sel, Scratch& s) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  uint32_t lo = 0xffffffffu, hi = 0;
   int c = 0;
-  for (int i = i0; i < i1; ++i) c += keys[i] != 0;
-  int valid;
-  block_excl_scan(c, s, &valid);
-  uint32_t tau = 1;   // select every key >= tau ...
-  int need_eq = 0x7fffffff;  // ... taking at most need_eq keys equal to tau (in index order)
-  if (valid > W) {
-    uint32_t prefix = 0, pmask = 0;
-    int rem = W;
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
-      for (int b = threadIdx.x; b < 256; b += NT) s.hist[b] = 0;
-      __syncthreads();
-      for (int i = i0; i < i1; ++i) {
+  for (int i = tid; i < n; i += NT) {
+    const uint32_t k = keys[i];
+    if (k != 0) {
+      lo = min(lo, k);
+      hi = max(hi, k);
+      ++c;
+    }
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) {
+    s.wlo[w] = lo;
+    s.whi[w] = hi;
+    s.wsum[w] = c;
+  }
+  if (tid < 256) s.hist[tid] = 0;
+  if (tid == 0) s.misc[2] = 0;
+  __syncthreads();
+  lo = __reduce_min_sync(0xffffffffu, s.wlo[lane]);
+  hi = __reduce_max_sync(0xffffffffu, s.whi[lane]);
+  const int valid = __reduce_add_sync(0xffffffffu, s.wsum[lane]);
+  const int m = min(W, valid);
+  // narrow [lo, hi], which holds the W-th best (as its rem-th), until it and all above it fit `cap`
+  const int cap = min(CAND, max(64, 2 * W));
+  int rem = W;
+  bool ties = false;   // more keys equal lo = hi than fit
+  if (valid > cap) {
+    for (;;) {
+      const int shift = max(0, 24 - __clz(hi - lo));   // 256 bins over [lo, hi]
+      for (int i = tid; i < n; i += NT) {
         const uint32_t k = keys[i];
-        if (k != 0 && (k & pmask) == prefix) atomicAdd(&s.hist[(k >> shift) & 255u], 1);
+        if (k != 0 && k >= lo && k <= hi) atomicAdd(&s.hist[(k - lo) >> shift], 1);
       }
       __syncthreads();
-      if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        // lane covers bins 255-8*lane .. 248-8*lane (descending)
+      if (w == 0) {
+        // lane l covers bins 255 - 8l .. 248 - 8l (descending)
+        const int4 q1 = reinterpret_cast<const int4*>(s.hist)[2 * (31 - lane) + 1];
+        const int4 q0 = reinterpret_cast<const int4*>(s.hist)[2 * (31 - lane)];
+        const int v[8] = {q1.w, q1.z, q1.y, q1.x, q0.w, q0.z, q0.y, q0.x};
         int loc = 0;
-        for (int j = 0; j < 8; ++j) loc += s.hist[255 - 8 * lane - j];
-        int inc = loc;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) loc += v[j];
+        int cum = loc;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, inc, o);
-          if (lane >= o) inc += y;
+          const int y = __shfl_up_sync(0xffffffffu, cum, o);
+          if (lane >= o) cum += y;
         }
-        const int exc = inc - loc;
-        if (exc < rem && rem <= inc) {
-          int cum = exc;
-          for (int j = 0; j < 8; ++j) {
-            const int b = 255 - 8 * lane - j;
-            if (cum + s.hist[b] >= rem) {
-              s.misc[0] = b;
-              s.misc[1] = rem - cum;
-              break;
-            }
-            cum += s.hist[b];
+        cum -= loc;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          if (cum < rem && rem <= cum + v[j]) {
+            s.misc[0] = 255 - 8 * lane - j;
+            s.misc[1] = rem - cum;
+            s.misc[3] = v[j];
           }
+          cum += v[j];
         }
       }
       __syncthreads();
-      const uint32_t b = (uint32_t)s.misc[0];
+      lo += (uint32_t)s.misc[0] << shift;
+      hi = lo + min(hi - lo, (1u << shift) - 1u);
       rem = s.misc[1];
-      prefix |= b << shift;
-      pmask |= 0xFFu << shift;
+      if (W - rem + s.misc[3] <= cap) break;
+      if (lo == hi) {
+        ties = true;
+        break;
+      }
+      if (tid < 256) s.hist[tid] = 0;
       __syncthreads();
     }
-    tau = prefix;
-    need_eq = rem;
   }
-  // rank of each tau-equal key among the tau-equal keys (index order)
-  int e = 0;
-  for (int i = i0; i < i1; ++i) e += keys[i] == tau;
-  int etot;
-  int ebefore = block_excl_scan(e, s, &etot);
-  // final flags and in-order compaction into tmp
-  int f = 0;
-  {
-    int er = ebefore;
-    for (int i = i0; i < i1; ++i) {
-      const uint32_t k = keys[i];
-      if (k == 0) continue;
-      if (k > tau) ++f;
-      else if (k == tau) {
-        if (er < need_eq) ++f;
-        ++er;
-      }
-    }
+  // the candidates: every key from lo up (of too many equal ones: the first `rem`)
+  auto put = [&](uint32_t k, int i) { s.cand[atomicAdd(&s.misc[2], 1)] = (unsigned long long)k << 32 | (uint32_t)~i; };
+  for (int i = tid; i < n; i += NT) {
+    const uint32_t k = keys[i];
+    if (k != 0 && k >= lo && !(ties && k == lo)) put(k, i);
   }
-  int m;
-  int pos = block_excl_scan(f, s, &m);
-  {
-    int er = ebefore;
-    for (int i = i0; i < i1; ++i) {
-      const uint32_t k = keys[i];
-      if (k == 0) continue;
-      bool take = false;
-      if (k > tau) take = true;
-      else if (k == tau) {
-        take = er < need_eq;
-        ++er;
-      }
-      if (take) tmp[pos++] = i;
-    }
+  if (ties) {
+    const int per = (n + NT - 1) / NT, i0 = tid * per, i1 = min(n, i0 + per);
+    int e = 0, etot;
+    for (int i = i0; i < i1; ++i) e += keys[i] == lo;
+    int er = block_excl_scan(e, s, &etot);
+    for (int i = i0; i < i1; ++i)
+      if (keys[i] == lo && er++ < rem) put(lo, i);
   }
   __syncthreads();
-  // rank the m selected by (key desc, index asc)
-  if (threadIdx.x < m) {
-    const int idx = tmp[threadIdx.x];
-    const uint32_t k = keys[idx];
+  // rank: four threads per candidate
+  const int nc = s.misc[2], mine = tid >> 2;
+  static_assert(NT == 4 * CAND, "four threads per candidate");
+  if ((w << 3) < nc) {
+    const unsigned long long x = mine < nc ? s.cand[mine] : ~0ull;
     int r = 0;
-    for (int j = 0; j < m; ++j) {
-      const int o = tmp[j];
-      const uint32_t ko = keys[o];
-      r += (ko > k) || (ko == k && o < idx);
-    }
-    sel[r] = idx;
+    for (int j = tid & 3; j < nc; j += 4) r += s.cand[j] > x;
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    if ((tid & 3) == 0 && mine < nc && r < W) sel[r] = (int)~(uint32_t)x;
   }
   __syncthreads();
   return m;
 }
 
 __device__ __forceinline__ int trie_child(const TreeDev& t, int x, int c) {
-  const uint32_t* mk = t.trie_mask + (size_t)x * 8;
-  int r = 0;
-  for (int w = 0; w < (c >> 5); ++w) r += __popc(mk[w]);
-  r += __popc(mk[c >> 5] & ((1u << (c & 31)) - 1u));
-  return t.trie_child[x] + r;
+  const uint4* mk = reinterpret_cast<const uint4*>(t.trie_mask + (size_t)x * 8);
+  const uint4 m0 = mk[0], m1 = mk[1];
+  const uint32_t v[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+  int r = t.trie_child[x];
+#pragma unroll
+  for (int w = 0; w < 8; ++w)
+    r += __popc(w < (c >> 5) ? v[w] : w == (c >> 5) ? v[w] & ((1u << (c & 31)) - 1u) : 0u);
+  return r;
 }
 
 // One warp: constrained log-probs of the valid children of trie node `tn`, given the 256 logits of
@@ -291,7 +307,7 @@ __device__ void write_out(const TreeDev& t, const VerifyOut& o, int K, int u, in
 __global__ void __launch_bounds__(NT) draft_level_kernel(TreeDev t, int lvl, int N, int relaxed, uint64_t seed) {
   extern __shared__ uint8_t sm[];
   __shared__ Scratch s;
-  __shared__ int sel[256], tmp[256];
+  __shared__ int sel[CAND];
   const int u = blockIdx.x;
   pdl_launch_dependents();
   pdl_wait();
@@ -324,7 +340,7 @@ __global__ void __launch_bounds__(NT) draft_level_kernel(TreeDev t, int lvl, int
     }
   }
   __syncthreads();
-  const int m = block_select(keys, n, N, sel, tmp, s);
+  const int m = block_select(keys, n, N, sel, s);
   const int off = level_off(t, lvl);
   const int depth = d + lvl;
   for (int r = threadIdx.x; r < t.slots_lvl; r += NT) {
@@ -363,10 +379,11 @@ __global__ void __launch_bounds__(NT) draft_level_kernel(TreeDev t, int lvl, int
 __global__ void __launch_bounds__(NT) verify_strict_kernel(TreeDev t, int K, VerifyOut o, int probe) {
   extern __shared__ uint8_t sm[];
   __shared__ Scratch s;
-  __shared__ int sel[256], tmp[256];
+  __shared__ int sel[CAND];
   __shared__ int yp_node[256];
   __shared__ float yp_sp[256];
-  __shared__ int match[256];
+  __shared__ uint16_t match[256];     // slot of the drafted node, kNone: none
+  __shared__ uint16_t drafted[256];   // parent's rank in its level (< 128: shared memory) * 256 + code of each drafted node
   __shared__ int n_yp, all_ok;
   const int u = blockIdx.x;
   pdl_launch_dependents();
@@ -388,6 +405,12 @@ __global__ void __launch_bounds__(NT) verify_strict_kernel(TreeDev t, int K, Ver
   int a = 0, adv = 0, m = 0;
   for (int j = 1; j <= last; ++j) {
     const int n = n_yp * TREE_CODES;
+    const int off = level_off(t, j), poff = level_off(t, j - 1);
+    const int nq = j <= g ? t.cnt[u * (t.max_levels + 1) + j] : 0;
+    for (int i = threadIdx.x; i < nq; i += NT) {
+      const int c = t.code[base + off + i];
+      drafted[i] = c >= 0 && c < TREE_CODES ? (uint16_t)(t.prank[base + off + i] * TREE_CODES + c) : kNone;
+    }
     for (int p = warp; p < n_yp; p += NW) {
       const int node = yp_node[p];
       const float* row = t.logits_t + (size_t)t.lg_t[node] * ITEM_ROWS + (d + j - 1) * TREE_CODES;
@@ -402,30 +425,33 @@ __global__ void __launch_bounds__(NT) verify_strict_kernel(TreeDev t, int K, Ver
       }
     }
     __syncthreads();
-    m = block_select(keys, n, K, sel, tmp, s);
+    m = block_select(keys, n, K, sel, s);
     if (j > g) {  // all drafted levels accepted: Y^p_{g+1} is the output
       a = g;
       adv = g + 1;
       break;
     }
     // is every selected (parent, code) a drafted node of level j?
-    const int off = level_off(t, j), poff = level_off(t, j - 1);
-    const int nq = t.cnt[u * (t.max_levels + 1) + j];
     if (threadIdx.x == 0) all_ok = 1;
     __syncthreads();
-    if (threadIdx.x < m) {
-      const int idx = sel[threadIdx.x];
-      const int pnode = yp_node[idx >> 8], c = idx & 255;
-      int f = -1;
-      for (int i = 0; i < nq; ++i) {
-        const size_t nd = base + off + i;
-        if (t.code[nd] == c && (int)(base + poff + t.prank[nd]) == pnode) {
-          f = (int)nd;
-          break;
-        }
+    if ((threadIdx.x >> 2) < (m + 7 & ~7)) {   // four threads per selected pair (whole warps)
+      const int r = threadIdx.x >> 2;
+      int f = 0x7fffffff;
+      if (r < m) {
+        const int idx = sel[r];
+        const int want = (yp_node[idx >> 8] - (int)base - poff) * TREE_CODES + (idx & 255);
+        for (int i = threadIdx.x & 3; i < nq; i += 4)
+          if (drafted[i] == want) {
+            f = i;
+            break;
+          }
       }
-      match[threadIdx.x] = f;
-      if (f < 0) atomicAnd(&all_ok, 0);
+      f = min(f, __shfl_xor_sync(0xffffffffu, f, 1));
+      f = min(f, __shfl_xor_sync(0xffffffffu, f, 2));
+      if (r < m && (threadIdx.x & 3) == 0) {
+        match[r] = f < nq ? (uint16_t)f : kNone;
+        if (f >= nq) all_ok = 0;
+      }
     }
     __syncthreads();
     if (probe && all_ok) {
@@ -442,9 +468,10 @@ __global__ void __launch_bounds__(NT) verify_strict_kernel(TreeDev t, int K, Ver
     if (threadIdx.x < m) nsp = score[sel[threadIdx.x]];
     __syncthreads();
     if (threadIdx.x < m) {
-      yp_node[threadIdx.x] = match[threadIdx.x];
+      const int nd = (int)base + off + match[threadIdx.x];
+      yp_node[threadIdx.x] = nd;
       yp_sp[threadIdx.x] = nsp;
-      t.sp[match[threadIdx.x]] = nsp;
+      t.sp[nd] = nsp;
     }
     if (threadIdx.x == 0) n_yp = m;
     __syncthreads();
@@ -485,7 +512,7 @@ __global__ void __launch_bounds__(NT) verify_relaxed_kernel(TreeDev t, int K, Ve
                                                             int probe) {
   extern __shared__ uint8_t sm[];
   __shared__ Scratch s;
-  __shared__ int sel[256], tmp[256];
+  __shared__ int sel[CAND];
   __shared__ int accd[256];     // accepted drafted slots, draft order
   __shared__ int outc[256];     // output candidate indices
   const int u = blockIdx.x;
@@ -534,7 +561,7 @@ __global__ void __launch_bounds__(NT) verify_relaxed_kernel(TreeDev t, int K, Ve
                                     : ordkey(v + gumbel(draw_u32(seed, STREAM_RESAMPLE, lvl_abs, step, u, i)));
       }
       __syncthreads();
-      nout = block_select(keys, n, K, sel, tmp, s);
+      nout = block_select(keys, n, K, sel, s);
       if (threadIdx.x < nout) outc[threadIdx.x] = sel[threadIdx.x];
       a = g;
       adv = g + 1;
@@ -606,12 +633,12 @@ __global__ void __launch_bounds__(NT) verify_relaxed_kernel(TreeDev t, int K, Ve
         for (int q = 0; q < na; ++q) r += (wsub[q] < w) || (wsub[q] == w && q < (int)threadIdx.x);
         if (r < K) {
           const size_t node = base + off + accd[threadIdx.x];
-          tmp[r] = t.prank[node] * TREE_CODES + t.code[node];
+          sel[r] = t.prank[node] * TREE_CODES + t.code[node];
         }
       }
       __syncthreads();
       mm = min(K, na);
-      if (threadIdx.x < mm) outc[threadIdx.x] = tmp[threadIdx.x];
+      if (threadIdx.x < mm) outc[threadIdx.x] = sel[threadIdx.x];
       nout = mm;
       a = g;
       adv = g;
@@ -638,7 +665,7 @@ __global__ void __launch_bounds__(NT) verify_relaxed_kernel(TreeDev t, int K, Ve
       keys[t.prank[node] * TREE_CODES + t.code[node]] = 0u;  // A is not resampled
     }
     __syncthreads();
-    int mm = block_select(keys, n, need, sel, tmp, s);
+    int mm = block_select(keys, n, need, sel, s);
     if (threadIdx.x < na) {
       const size_t node = base + off + accd[threadIdx.x];
       outc[threadIdx.x] = t.prank[node] * TREE_CODES + t.code[node];
@@ -656,7 +683,7 @@ __global__ void __launch_bounds__(NT) verify_relaxed_kernel(TreeDev t, int K, Ve
       __syncthreads();
       for (int q = threadIdx.x; q < na + mm; q += NT) keys[outc[q]] = 0u;
       __syncthreads();
-      const int m2 = block_select(keys, n, need - mm, sel, tmp, s);
+      const int m2 = block_select(keys, n, need - mm, sel, s);
       if (threadIdx.x < m2) outc[na + mm + threadIdx.x] = sel[threadIdx.x];
       mm += m2;
       __syncthreads();

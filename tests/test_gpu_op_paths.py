@@ -157,3 +157,52 @@ def test_full_lse_paths(ats, V, users, N, gamma):
     # fp32 logits (|x . w| up to ~30) and exponentials of them: a few units of 2^-23 of the largest logit
     assert float((got - ref).abs().max()) < 2e-5
     ctx.close()
+
+
+# the exact selection of a drafted level (score descending, index ascending): one histogram pass, several (an
+# outlier widens the range), none (few candidates), more equal keys than are ranked at once, infinite scores
+@pytest.mark.parametrize("N", [1, 5, 40, 100])
+@pytest.mark.parametrize("kind", ["spread", "outlier", "equal", "three", "inf", "few"])
+def test_selection_paths(ats, kind, N):
+    from types import SimpleNamespace
+    d, f, V = 64, 128, 1024
+    w = {"embed": _randn((V, d), 1), "lm_head": _randn((V, d), 2, 0.4), "final_norm": _randn((d,), 3, 0.1) + 1}
+    for name, shape in (("attn_norm", (d,)), ("mlp_norm", (d,)), ("wqkv", (3 * d, d)), ("wo", (d, d)),
+                        ("wgate_up", (2 * f, d)), ("wdown", (d, f))):
+        w["layers.0." + name] = _randn(shape, 4 + len(name), 0.1)
+    spec = SimpleNamespace(n_layers=1, d_model=d, n_heads=2, d_ffn=f, vocab=V, rms_eps=1e-6, rope_theta=1e4)
+    n = 7 if kind == "few" else 256
+    items = np.zeros((n * n, 4), np.int32)
+    items[:, 0], items[:, 1] = np.repeat(np.arange(n), n), np.tile(np.arange(n), n)
+    rng = np.random.default_rng(N)
+    # logits of the two levels, the same for every parent: different sums differ by 2^-8 at least, beyond fp32
+    # rounding, so the order of the sums is that of the scores
+    x = [rng.permutation(256) * 1.0, rng.permutation(256) / 256.0]
+    if kind == "outlier":
+        x = [1 + rng.permutation(256) / 256.0, rng.permutation(256) * 1.0]
+        x[0][3] = x[1][200] = -10000.0
+    elif kind == "equal":
+        x = [np.full(256, 1.25)] * 2
+    elif kind == "three":
+        x = [np.array([0.0, 1.0, 3.0])[rng.integers(0, 3, 256)] for _ in range(2)]
+    elif kind == "inf":
+        for v in x:
+            v[rng.permutation(256)[:250]] = -np.inf
+    ctx = ats.Context(spec, w, spec, w, items, 0, max_users=1, max_prompt=8, max_K=1, max_N=N, max_gamma=2)
+    o = ats.opts(1, N, 2)
+    ctx.prefill(torch.arange(8, dtype=torch.int32, device="cuda"), [0, 8])
+    ctx.begin_step(o)
+    beams, score = [()], np.zeros(1)
+    for lvl in range(2):
+        tree = ctx.debug_tree(2)
+        width = tree["slots_in"] if lvl == 0 else tree["slots_lvl"]
+        ctx.draft_step_logits(o, ats.STRICT, np.tile(np.tile(x[lvl], 4).astype(np.float32), (1, width, 1)))
+        s = (score[:, None] + x[lvl][None, :n]).reshape(-1)
+        order = np.lexsort((np.arange(s.size), -s))[:N]
+        beams, score = [beams[i // n] + (i % n,) for i in order], s[order]
+        tree = ctx.debug_tree(2)
+        off = tree["slots_in"] + lvl * tree["slots_lvl"]
+        assert tree["count"][0, lvl + 1] == len(order)
+        got = [tuple(int(c) for c in q if c >= 0) for q in tree["path"][0, off:off + len(order)]]
+        assert got == beams
+    ctx.close()
