@@ -62,7 +62,7 @@ struct Fail {
 struct ModelRt {
   bool present = false;
   bool per_op = false;   // this model's forward runs one kernel per op (else one persistent launch)
-  int grid = 0;          // CTAs of its GEMM work splits (both schedules, so both give the same bits)
+  int grid = 0;          // CTAs of the current forward's GEMM work splits (both schedules, so both give the same bits)
   int cps = 2;           // prefix pages per attention split of its tree forwards (fixed per context)
   int layers = 0, d = 0, H = 0, hd = 0, ffn = 0, V = 0;
   float eps = 1e-6f, theta = 1e4f;
@@ -106,6 +106,25 @@ struct ModelRt {
   int* plan_blk = nullptr;   // qt_* / user_splits / rows_sel of the current forward, packed
   int max_qt = 0;
 };
+
+// CTAs of a forward of T tokens.  One token tile (256 tokens): min(SMs, gate/up weight tiles), so that a
+// small model takes one whole gate/up tile per CTA with no split sums, and every grid barrier spans fewer
+// CTAs (4 layers, 48 tiles, 128 tokens, us on 48 / 96 / 152 CTAs: 184 / 213 / 262).  More token tiles give
+// work to more CTAs: short gate/up tiles (<= 16 k-blocks) still whole, as evenly as that goes (the sum of a
+// split tile costs as much as the tile), long ones on every SM.  us on the weight tiles' count of CTAs ->
+// here: the 4-layer model, 512 tokens 297 -> 250 (152 CTAs: 345), 1000 536 -> 342 (403), 3000 1254 -> 566
+// (686), 4000 1544 -> 769 (814); 2 layers of 2048 (88 tiles of 32 k-blocks), 512 tokens 252 -> 234, 1000 455
+// -> 351 (118 whole-tile CTAs: 405), 4000 1400 -> 910; the 2-layer d 128 model (8 tiles), 1000 tokens 306 ->
+// 142, 4000 1012 -> 161 (the attention's items ask for at least 64 there: 32 CTAs 151 at 1000 tokens).
+int forward_ctas(const ModelRt& m, int T, int sms) {
+  const int weight_tiles = 2 * m.ffn / 128, tiles = weight_tiles * std::max(1, (T + 255) / 256);
+  int G = tiles;
+  if (T > 256 && m.d / 64 <= 16) {
+    const int waves = (tiles + sms - 1) / sms;
+    G = std::max((tiles + waves - 1) / waves, 64);
+  }
+  return std::max(1, std::min(sms, G));
+}
 
 struct UserState {
   int P = 0;          // prompt length
@@ -423,7 +442,7 @@ void alloc_model(atspeed_ctx* c, ModelRt& m) {
   const int pages = c->prefix_pages_per_user;
   {
     // the grid the model's forward will run on (as set with the schedule) and its split size
-    const int grid = std::max(1, std::min(gemm_grid_size(c->device), 2 * m.ffn / 128));
+    const int grid = forward_ctas(m, 1, gemm_grid_size(c->device));
     m.cps = attention_pages_per_split(L, m.H, grid);
   }
   m.max_splits = std::max(1, (pages + m.cps - 1) / m.cps);
@@ -639,6 +658,7 @@ void forward(atspeed_ctx* c, ModelRt& m, const FwdPlan& p, cudaStream_t st) {
     set_err(c, "forward of %d tokens exceeds capacity %d", T, m.Tcap);
     throw Fail{ATSPEED_E_SHAPE};
   }
+  m.grid = forward_ctas(m, T, c->fwd_grid);
   const int nqt = (int)p.qt_t0.size();
   if (nqt > m.max_qt || (int)p.splits.size() > c->lim.max_users || (int)p.out_rows.size() > m.Tcap) {
     set_err(c, "forward plan exceeds capacity (%d query tiles, %zu users, %zu rows)", nqt, p.splits.size(),
@@ -1486,15 +1506,12 @@ atspeed_status atspeed_create(const atspeed_model_desc* target, const atspeed_mo
     c->fwd_grid = c->gemm_grid;  // one persistent CTA per SM
     {
       // Schedule of a model's forward: one persistent launch; ATSPEED_FORWARD=per_op runs one kernel
-      // per op instead (same bits).  GEMM work splits run over min(SMs, gate/up weight tiles) CTAs:
-      // a small model (the 4-layer draft: 48 tiles) then takes one whole gate/up tile per CTA with
-      // no split sums, and every phase's grid barrier spans fewer CTAs; a 7B-shape model (172 tiles)
-      // takes the whole GPU.
+      // per op instead (same bits).
       const char* fm = getenv("ATSPEED_FORWARD");
       c->forward_mode = (fm && strcmp(fm, "persistent") == 0) ? 1 : (fm && strcmp(fm, "per_op") == 0) ? 2 : 0;
       for (ModelRt* mr : {&c->tgt, &c->drf}) {
         mr->per_op = c->forward_mode == 2;
-        mr->grid = std::max(1, std::min(c->fwd_grid, 2 * mr->ffn / 128));
+        mr->grid = forward_ctas(*mr, 1, c->fwd_grid);
       }
     }
     {
