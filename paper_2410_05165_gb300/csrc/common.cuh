@@ -237,10 +237,10 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
         : "memory");
 }
 
-// Arrive on an mbarrier (CG = 2: at this offset in both CTAs) once every previously issued
-// tcgen05.mma of this thread has completed.
+// Arrive on an mbarrier (CG = 2: at this offset in both CTAs, the cluster ranks of `pair`) once every
+// previously issued tcgen05.mma of this thread has completed.
 template <int CG = 1>
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+__device__ __forceinline__ void tc_commit(uint64_t* bar, uint16_t pair = 3) {
   if constexpr (CG == 1)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
@@ -248,7 +248,7 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
             smem_u32(bar)),
-        "h"((uint16_t)3)
+        "h"(pair)
         : "memory");
 }
 

@@ -2,7 +2,7 @@
 // small prefill shapes).  Same product and operands as gemm.cu (weight rows are the MMA's M, tokens
 // its N), another decomposition:
 //
-//   * one cluster of C CTAs (C <= 8) per tile of 128 weight rows x BN tokens; CTA r streams the r-th
+//   * one cluster of C CTAs (C <= 8; or CTA pairs) per tile of 128 weight rows x BN tokens; CTA r streams the r-th
 //     share of the k-blocks through its TMA ring into two TMEM accumulators, half of the share each (the
 //     tensor core rounds towards zero, so the error grows with the length of an accumulation);
 //   * the partial sums meet in distributed shared memory: the tile's 16-token groups are dealt out to
@@ -20,11 +20,18 @@
 // that the second wave's CTAs run beside the first's.  Two per SM and larger clusters were slower where
 // one wave is enough: half the copies in flight per CTA and more partials to exchange.
 //
+// Long shares run as CTA pairs (CG = 2): two CTAs of 128 weight rows each and half of the tokens' operand
+// issue one tcgen05.mma of 256 rows.  The order of every sum is the same; the tokens' operand is written
+// to and read from shared memory once per pair, where its 128 bytes a clock bind the 256-token tile (48 KB in
+// and 48 KB out per k-block of 512 clocks of MMA), and the ring is half as deep again (us, 256-token tiles:
+// [4096 x 11008] x 512 40.4 -> 34.4, x 960 66.9 -> 55.3, [12288 x 4096] x 200 29.4 -> 24.6, [22016 x 4096] x 200
+// 53.1 -> 46.2; 128: [19456 x 4096] x 120 29.9 -> 28.6).
+//
 // Measured against the stream-K kernel / two narrow CTAs per SM (us, GB300): [12288 x 4096] x 120 tokens
-// 32.1 / 23.7 -> 22.7 (4.5 TB/s), x 200 31.4 -> 29.4 (narrow), x 10 20.1 -> 21.4 (narrow; the one loss: an SM
+// 32.1 / 23.7 -> 22.7 (4.5 TB/s), x 200 31.4 -> 24.6 (narrow), x 10 20.1 -> 21.4 (narrow; the one loss: an SM
 // takes in 60 bytes per ns, and 96 of 152 are used), [4096 x 11008] x 120 31.4 / 24.7 -> 20.6, x 200 35.6
 // -> 25.7 (narrow), [4096 x 4096] x 120 23.3 / 16.2 -> 12.4, [768 x 768] x 10 9.4 / 6.5 -> 5.8, [4096 x 11008] x
-// 512 56.6 / 46.3 -> 40.7, x 960 90.2 / 72.6 -> 67.0.
+// 512 56.6 / 46.3 -> 34.4, x 960 90.2 / 72.6 -> 55.3.
 // Error against fp64 (relative, stream-K kernel / here): [4096 x 11008] 2.3e-6 / 1.4e-6, [4096 x 4096] 7.9e-7 /
 // 4.7e-7, [768 x 768] 0.9e-7 / 1.1e-7, [22016 x 4096] 4.2e-6 / 4.4e-6.
 //
@@ -50,13 +57,13 @@ constexpr int GROUP = 16;                            // tokens of an exchange gr
 constexpr int GROUP_FLOATS = GROUP * GEMM_BM;        // one CTA's partial of a group: [token/4][row][4]
 constexpr int STG_LD = GEMM_BM + 4;                  // staging row of one token (SwiGLU), floats
 
-template <int BN>
+template <int BN, int CG>
 struct KCfg {
   static constexpr int A_BYTES = GEMM_BM * 128;
-  static constexpr int B_BYTES = BN * 128;
+  static constexpr int B_BYTES = BN / CG * 128;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   // copies in flight: two CTAs per SM, or one ("wide")
-  static constexpr int STAGES = BN >= 256 ? 2 : BN >= 128 ? 3 : BN >= 64 ? 4 : 5;
+  static constexpr int STAGES = CG == 2 ? (BN >= 256 ? 3 : 4) : BN >= 256 ? 2 : BN >= 128 ? 3 : BN >= 64 ? 4 : 5;
   static constexpr int WIDE_STAGES = (232448 - 1024 - 256) / STAGE_BYTES;
   // after the last MMA: (wide) receive area, a CTA owns at most ceil(groups / C) groups, each with C - 1
   // received partials; then a staging buffer per warpgroup
@@ -99,11 +106,11 @@ __device__ __forceinline__ void ld_group(uint32_t addr, uint32_t second, float (
   }
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, int CG>
 __global__ void __launch_bounds__(THREADS, 2)
     gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const KcParams p) {
-  using C = KCfg<BN>;
+  using C = KCfg<BN, CG>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int stages = p.wide ? C::WIDE_STAGES : C::STAGES;
@@ -114,9 +121,11 @@ __global__ void __launch_bounds__(THREADS, 2)
   int* failed = reinterpret_cast<int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nc = p.C, rank = nc > 1 ? (int)cluster_ctarank() : 0;
-  const int tile = blockIdx.x / nc;
-  const int m_tile = tile / p.n_tiles, n_tile = tile % p.n_tiles;
+  // rank: the k-share; half: the CTA of a pair (CG = 2), whose 128 of the pair's 256 weight rows it takes
+  const int nc = p.C, crank = nc * CG > 1 ? (int)cluster_ctarank() : 0, rank = crank / CG, half = crank % CG;
+  const int lead = crank - half;   // cluster rank of the pair's issuing CTA
+  const int tile = blockIdx.x / (nc * CG);
+  const int m_tile = tile / p.n_tiles * CG + half, n_tile = tile % p.n_tiles;
   const int k0 = rank * p.kb / nc, k1 = (rank + 1) * p.kb / nc;   // this CTA's k-blocks (never empty: C <= kb)
   const int k2 = p.wide ? k0 + (k1 - k0 + 1) / 2 : k1;             // the second accumulator's first
 
@@ -130,11 +139,12 @@ __global__ void __launch_bounds__(THREADS, 2)
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, (uint32_t)(p.wide ? 2 * BN : BN));
-    tmem_relinquish();
+    tmem_alloc<CG>(tmem_slot, (uint32_t)(p.wide ? 2 * BN : BN));
+    tmem_relinquish<CG>();
   }
   tc_fence_before();
   __syncthreads();
+  if (CG == 2) cluster_sync();   // the other CTA's barriers are initialised too
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -160,10 +170,12 @@ __global__ void __launch_bounds__(THREADS, 2)
           break;
         }
         uint8_t* sa = smem + stage * C::STAGE_BYTES;
-        mbar_arrive_expect_tx(&full[stage], C::STAGE_BYTES);
-        tma_load_2d(sa, &tmA, &full[stage], k * GEMM_BK, r0, pol_w);
-        tma_load_2d(sa + 8192, &tmA, &full[stage], k * GEMM_BK, r1, pol_w);
-        tma_load_2d(sa + C::A_BYTES, &tmB, &full[stage], k * GEMM_BK, n_tile * BN, pol_x);
+        // (a pair's copies all count on the issuing CTA's barrier)
+        const uint32_t fb = CG == 2 ? mapa_u32(&full[stage], (uint32_t)lead) : smem_u32(&full[stage]);
+        if (half == 0) mbar_arrive_expect_tx(&full[stage], CG * C::STAGE_BYTES);
+        tma_load_2d_cg<CG>(sa, &tmA, fb, k * GEMM_BK, r0, pol_w);
+        tma_load_2d_cg<CG>(sa + 8192, &tmA, fb, k * GEMM_BK, r1, pol_w);
+        tma_load_2d_cg<CG>(sa + C::A_BYTES, &tmB, fb, k * GEMM_BK, n_tile * BN + half * (BN / CG), pol_x);
         if (++stage == stages) {
           stage = 0;
           phase ^= 1u;
@@ -171,9 +183,10 @@ __global__ void __launch_bounds__(THREADS, 2)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (lane == 0 && half == 0) {
       // ------------------------------------------------------------------ MMA issuer
-      constexpr uint32_t idesc = idesc_bf16_f32(GEMM_BM, BN);
+      constexpr uint32_t idesc = idesc_bf16_f32(CG * GEMM_BM, BN);
+      const uint16_t pair = (uint16_t)(3u << lead);
       int stage = 0;
       uint32_t phase = 0;
       for (int k = k0; k < k1; ++k) {
@@ -186,15 +199,15 @@ __global__ void __launch_bounds__(THREADS, 2)
         const uint64_t ad = smem_desc_sw128(sa), bd = smem_desc_sw128(sa + C::A_BYTES);
 #pragma unroll
         for (int kk = 0; kk < GEMM_BK / 16; ++kk)
-          tc_mma_bf16(k < k2 ? tmem_base : tmem_base + BN, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc,
+          tc_mma_bf16<CG>(k < k2 ? tmem_base : tmem_base + BN, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc,
                       ((k != k0 && k != k2) || kk > 0) ? 1u : 0u);
-        tc_commit(&empty[stage]);
+        tc_commit<CG>(&empty[stage], pair);
         if (++stage == stages) {
           stage = 0;
           phase ^= 1u;
         }
       }
-      tc_commit(tfull);   // (also after a failure: nothing may run when TMEM is released)
+      tc_commit<CG>(tfull, pair);   // (also after a failure: nothing may run when TMEM is released)
     }
   }
   __syncwarp();   // (the other lanes of the role warps do not poll beside their lane 0)
@@ -215,7 +228,8 @@ __global__ void __launch_bounds__(THREADS, 2)
   const uint32_t tb = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
   float* recv = reinterpret_cast<float*>(smem);
   float* stg = reinterpret_cast<float*>(smem + C::stg_off(p.wide) + (wg & 1) * C::STG_BYTES);
-  const int nvalid = min(BN, a.T - n_tile * BN);
+  // (an odd last weight tile leaves a pair's second CTA without rows)
+  const int nvalid = CG == 1 || m_tile < p.m_tiles ? min(BN, a.T - n_tile * BN) : 0;
   const uint32_t second = k2 < k1 ? BN : 0;   // the second accumulator's columns
   if (nc > 1) cluster_sync();   // every CTA's ring is idle: it may receive partials
   const int ng = (nvalid + GROUP - 1) / GROUP;   // groups: owner = group % C
@@ -229,7 +243,7 @@ __global__ void __launch_bounds__(THREADS, 2)
         ld_group(tb + g * GROUP, second, r);
         // slot of (group, source) in the owner's receive area
         const int slot = (g / nc) * (nc - 1) + (rank < owner ? rank : rank - 1);
-        const uint32_t dst = mapa_u32(recv + slot * GROUP_FLOATS + m * 4, (uint32_t)owner);
+        const uint32_t dst = mapa_u32(recv + slot * GROUP_FLOATS + m * 4, (uint32_t)(owner * CG + half));
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           st_cluster_f4(dst + j * (GEMM_BM * 16), make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]));
@@ -329,39 +343,41 @@ __global__ void __launch_bounds__(THREADS, 2)
   }
   tc_fence_before();
   __syncthreads();
+  if (CG == 2) cluster_sync();   // neither CTA of a pair leaves before the other is done
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, (uint32_t)(p.wide ? 2 * BN : BN));
+    tmem_dealloc<CG>(tmem_base, (uint32_t)(p.wide ? 2 * BN : BN));
   }
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, int CG>
 cudaError_t launch_t(const CUtensorMap& ma, const CUtensorMap& mb, const KcParams& kp, cudaStream_t st) {
+  using C = KCfg<BN, CG>;
   static std::atomic<unsigned long long> attr_done{0};
-  const cudaError_t e = smem_attr_once(attr_done, gemm_cluster_kernel<BN, EPI>, KCfg<BN>::smem(true));
+  const cudaError_t e = smem_attr_once(attr_done, gemm_cluster_kernel<BN, EPI, CG>, C::smem(true));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(kp.m_tiles * kp.n_tiles * kp.C));
+  cfg.gridDim = dim3((unsigned)((kp.m_tiles + CG - 1) / CG * kp.n_tiles * kp.C * CG));
   cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = KCfg<BN>::smem(kp.wide);
+  cfg.dynamicSmemBytes = C::smem(kp.wide);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)kp.C;
+  at[0].val.clusterDim.x = (unsigned)(kp.C * CG);
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = kp.C > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, gemm_cluster_kernel<BN, EPI>, ma, mb, kp);
+  cfg.numAttrs = kp.C * CG > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, gemm_cluster_kernel<BN, EPI, CG>, ma, mb, kp);
 }
 
-template <int BN>
+template <int BN, int CG>
 cudaError_t launch_bn(EpiKind e, const CUtensorMap& ma, const CUtensorMap& mb, const KcParams& kp, cudaStream_t st) {
   switch (e) {
-    case EPI_F32: return launch_t<BN, EPI_F32>(ma, mb, kp, st);
-    case EPI_RESID: return launch_t<BN, EPI_RESID>(ma, mb, kp, st);
-    case EPI_SWIGLU: return launch_t<BN, EPI_SWIGLU>(ma, mb, kp, st);
-    case EPI_LSE: return launch_t<BN, EPI_LSE>(ma, mb, kp, st);
+    case EPI_F32: return launch_t<BN, EPI_F32, CG>(ma, mb, kp, st);
+    case EPI_RESID: return launch_t<BN, EPI_RESID, CG>(ma, mb, kp, st);
+    case EPI_SWIGLU: return launch_t<BN, EPI_SWIGLU, CG>(ma, mb, kp, st);
+    case EPI_LSE: return launch_t<BN, EPI_LSE, CG>(ma, mb, kp, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -385,8 +401,8 @@ int cluster_size(long long tiles, int kb, int sms) {
 bool gemm_cluster_fits(const GemmArgs& a, int sms) {
   if (a.epi != EPI_F32 && a.epi != EPI_RESID && a.epi != EPI_SWIGLU && a.epi != EPI_LSE) return false;
   // One token tile: always (so that up to 256 tokens the k-split does not depend on the token count).
-  // More: while every tile has an SM of its own.  At the line (us, cluster / CTA pairs, K = 4096): 128 tiles
-  // ([8192] x 512 tokens) 29.7 / 41.2, 160 ([5120] x 1000) 47.5 / 51.6, 192 ([12288] x 512) 56.5 / 41.9.
+  // More: while every tile has an SM of its own.  At the line (us, here / gemm_pair.cu, K = 4096): 128 tiles
+  // ([8192] x 512 tokens) 26.0 / 41.2, 152 ([9728] x 512) 27.5 / 27.7, 192 ([12288] x 512) 56.5 / 41.9.
   if (a.T <= 256) return true;
   const long long m_tiles = a.epi == EPI_SWIGLU ? a.M / 128 : ((long long)a.M + 127) / 128;
   return m_tiles * ((a.T + 255) / 256) <= sms;
@@ -408,12 +424,21 @@ cudaError_t gemm_cluster_launch(const GemmArgs& a, unsigned int* err, int sms, c
   kp.err = err;
   CUtensorMap ma, mb;
   if (!gemm_make_map(&ma, a.W, a.K, a.M, 64, eb, el)) return kGemmMapError;
-  if (!gemm_make_map(&mb, a.X, a.K, a.X_rows, BN, eb, el)) return kGemmMapError;
+  // CTA pairs (the same sums) for long shares, while all clusters of 2 C CTAs still run at once.  At the
+  // lines (us, one CTA / pair): 256 tokens, C = 2 of 40 k-blocks 14.3 / 14.8 as C = 3, 1 of 4 7.2 / 7.7, 1 of 12
+  // 16.9 / 16.3, 1 of 64 30.1 / 25.5; 120 tokens, C = 1 of 12 k-blocks 11.5 / 12.6, of 32 14.1 / 14.5, of 64 with
+  // 128 weight tiles 27.7 / 26.4, 160 35.8 / 34.6, 258 47.5 / 48.1.
+  const long long tiles = (long long)kp.m_tiles * kp.n_tiles, pair_ctas = 2LL * ((kp.m_tiles + 1) / 2) * kp.n_tiles * kp.C;
+  const bool room = !kp.wide || pair_ctas <= (kp.C == 1 ? sms : sms * 9 / 10);
+  const bool pairs = BN == 256 ? kp.C <= 2 && kp.kb >= 8 * kp.C && room
+                               : BN == 128 && kp.C == 1 && kp.kb >= 48 && 2 * tiles <= 3 * sms && room;
+  if (!gemm_make_map(&mb, a.X, a.K, a.X_rows, pairs ? BN / 2 : BN, eb, el)) return kGemmMapError;
+  if (pairs) return BN == 128 ? launch_bn<128, 2>(a.epi, ma, mb, kp, stream) : launch_bn<256, 2>(a.epi, ma, mb, kp, stream);
   switch (BN) {
-    case 32: return launch_bn<32>(a.epi, ma, mb, kp, stream);
-    case 64: return launch_bn<64>(a.epi, ma, mb, kp, stream);
-    case 128: return launch_bn<128>(a.epi, ma, mb, kp, stream);
-    default: return launch_bn<256>(a.epi, ma, mb, kp, stream);
+    case 32: return launch_bn<32, 1>(a.epi, ma, mb, kp, stream);
+    case 64: return launch_bn<64, 1>(a.epi, ma, mb, kp, stream);
+    case 128: return launch_bn<128, 1>(a.epi, ma, mb, kp, stream);
+    default: return launch_bn<256, 1>(a.epi, ma, mb, kp, stream);
   }
 }
 

@@ -56,7 +56,8 @@ def test_gemm_paths(ats, M, K, T):
 
 
 @pytest.mark.parametrize("F,K,T", [(64, 64, 1), (192, 128, 16), (320, 512, 33), (1408, 1024, 128), (1024, 4096, 130),
-                                   (3072, 768, 257), (11008, 256, 250), (9728, 192, 40), (5632, 128, 700)])
+                                   (3072, 768, 257), (11008, 256, 250), (9728, 192, 40), (5632, 128, 700),
+                                   (6080, 128, 120), (9792, 128, 70), (960, 512, 400)])
 def test_swiglu_paths(ats, F, K, T):
     W, X = _randn((2 * F, K), F + K, 0.05), _x(T, K, T)
     g, u = (X[:T].double() @ W.double().T).split(F, 1)
@@ -66,8 +67,8 @@ def test_swiglu_paths(ats, F, K, T):
     assert bool(((out - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-4 * (g.abs() + u.abs() + 1)).all())
 
 
-def test_gemm_result_does_not_depend_on_the_token_count(ats):
-    M, K = 2304, 768
+@pytest.mark.parametrize("M,K", [(2304, 768), (8192, 512), (6400, 256), (20000, 256)])
+def test_gemm_result_does_not_depend_on_the_token_count(ats, M, K):
     W, X = _randn((M, K), 5), _x(256, K, 6)
     full = ats.op_gemm(W, X, 256)
     for T in (1, 16, 33, 100, 129, 200):
