@@ -55,6 +55,19 @@ atspeed_status run_gemm(cudaStream_t st, const GemmArgs& a, void* ws) {
   return gemm_status(gemm_pair_launch(a, s, grid, st, eb, sizeof eb));
 }
 
+// CTAs (prefix splits) per (query tile, head): as many of 4, 2, 1 as run at once (three CTAs per SM) and
+// leave each CTA pages enough.  One CTA without path keys writes its rows directly, so a short prefix is
+// not split then.  us, 1 / 2 / 4 CTAs, 128-wide heads: 128 pairs of 8 pages with path keys 21.8 / 18.1 / 25.5,
+// 256 of 8 26.6 / 32.7 / 42.0, 64 of 8 21.8 / 14.4 / 14.0, 64 of 5 17.1 / 12.9 / 13.9, 32 of 5 13.8 / 10.8 / 10.3;
+// causal without: 128 of 4 9.2 / 11.7 / 21.2, 256 of 8 17.5 / 22.2 / 36.8; 64-wide heads: 48 of 4 6.6 / 7.4 / 7.3,
+// 72 of 6 8.6 / 8.5 / 8.0, 192 of 16 19.6 / 16.9 / 19.5; 32-wide: 16 of 4 7.1 / 7.5 / 5.6.
+int attention_splits(long long pairs, int pages, bool paths, int sms) {
+  const long long room = 3LL * sms;
+  const int least4 = paths ? (8 * pairs <= 3LL * sms ? 4 : 8) : 4 * pairs <= sms ? 4 : 6;
+  if (4 * pairs <= room && pages >= least4) return 4;
+  return 2 * pairs <= room && pages >= (paths ? 2 : 8) ? 2 : 1;
+}
+
 // ---------------------------------------------------------------------------------------------
 // Allocation-free GEMM: its split-K scratch lives in a fixed device array of this library.
 // ---------------------------------------------------------------------------------------------
@@ -158,9 +171,6 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
   cudaStream_t st = (cudaStream_t)stream;
   const int pages = (P + ATT_PAGE - 1) / ATT_PAGE;
   const int nqt = (T + ATT_QTILE - 1) / ATT_QTILE;
-  // CTAs per (query tile, head): about two per SM in all (three fit), no more than pages to share
-  const long long pairs = (long long)nqt * n_heads, want = 2LL * current_grid();
-  const int S = pairs >= want || pages < 2 ? 1 : 2 * pairs >= want || pages < 4 ? 2 : 4;
   for (int p = 0; p < pages; ++p)
     if (h_pages[p] < 0 || (h_pages[p] + 1) * ATT_PAGE > cache_rows) return ATSPEED_E_ARG;
   for (int t = 0; t < T; ++t) {
@@ -172,6 +182,7 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
   }
   bool paths = false;
   for (int t = 0; h_n_path && t < T; ++t) paths |= h_n_path[t] > 0;
+  const int S = attention_splits((long long)nqt * n_heads, pages, paths, current_grid());
   const int d = n_heads * head_dim;
   CUtensorMap mk, mv;
   char eb[256];
