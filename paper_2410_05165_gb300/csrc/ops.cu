@@ -26,8 +26,7 @@ int current_grid() {
   return gemm_grid_size(dev);
 }
 
-GemmScratch scratch_from(void* ws) {
-  const int G = current_grid();
+GemmScratch scratch_from(void* ws, int G) {
   GemmScratch s;
   s.ws = static_cast<float*>(ws);
   s.ws_bytes = gemm_ws_bytes(G);
@@ -50,7 +49,7 @@ atspeed_status run_gemm(cudaStream_t st, const GemmArgs& a, void* ws) {
   if (!ws) return ATSPEED_E_ARG;
   char eb[256];
   const int grid = current_grid();
-  const GemmScratch s = scratch_from(ws);
+  const GemmScratch s = scratch_from(ws, grid);
   if (gemm_cluster_fits(a, grid)) return gemm_status(gemm_cluster_launch(a, s.err, grid, st, eb, sizeof eb));
   return gemm_status(gemm_pair_launch(a, s, grid, st, eb, sizeof eb));
 }
@@ -264,7 +263,7 @@ atspeed_status atspeed_op_gemm_noalloc(atspeed_stream stream, const void* d_W, c
 atspeed_status atspeed_op_status(atspeed_stream stream, void* d_ws) {
   unsigned int* word = nullptr;
   if (d_ws) {
-    word = scratch_from(d_ws).err;
+    word = scratch_from(d_ws, current_grid()).err;
   } else {
     void* base = noalloc_base();
     if (!base) return ATSPEED_E_CUDA;
