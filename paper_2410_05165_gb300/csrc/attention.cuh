@@ -49,7 +49,7 @@ struct AttnArgs {
   unsigned int* err;
 };
 
-// Encodes the K/V tensor maps for one layer's cache arena (box = 64 rows x min(head_dim, 64)).
+// Encodes the K/V tensor maps for one layer's cache arena (box = ATT_SUB rows x min(head_dim, 64)).
 bool attn_make_maps(const __nv_bfloat16* k_cache, const __half* v_cache, int rows, int d_model,
                     int head_dim, CUtensorMap* mk, CUtensorMap* mv, char* eb, size_t el);
 

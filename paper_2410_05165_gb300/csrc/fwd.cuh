@@ -15,7 +15,7 @@ namespace atspeed {
 // Tensor-map table layout (device memory, 64-byte aligned CUtensorMap entries):
 //   [l*4 + 0..3]    weights of layer l: wqkv, wo, wgate_up, wdown   (box 64 x 128, 128B swizzle;
 //                   wgate_up three-dimensional [gate | up][d_ffn][d], box 64 x 64 x 2)
-//   [4L + 2l + 0/1] K / V cache of layer l                          (box hd' x 64, attention)
+//   [4L + 2l + 0/1] K / V cache of layer l                          (box min(hd, 64) x 32, attention)
 //   [6L + 0]        item-code rows of the LM head                   (box 64 x 128)
 //   [6L + 1..3]     activations x, att, act, token tile 128         (box 64 x 128)
 //   [6L + 4..6]     activations x, att, act, token tile 256         (box 64 x 256)

@@ -1,6 +1,8 @@
 // Weight-streaming GEMM for sm_103a: TMA -> shared memory (128B swizzle) -> tcgen05.mma with the
 // fp32 accumulator in TMEM -> tcgen05.ld epilogue with fused QKV+RoPE+KV-store / SwiGLU /
-// residual-add (with the next RMSNorm's partial sums) / plain stores.
+// residual-add (with the next RMSNorm's partial sums) / plain stores.  The GEMM of the one-kernel-per-op
+// schedule (the persistent kernel's work split and epilogues: the same bits) and of the allocation-free
+// entry point; the other operators take gemm_cluster.cu and gemm_pair.cu.
 //
 // Decomposition ("stream-K"): the work units are (tile, 64-wide k-block) pairs, tile = (weight-row
 // tile of 128, token tile of BN), ordered weight-tile-major.  A persistent grid of one CTA per SM
