@@ -274,6 +274,91 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// One thread of a converged warp.  The producers and the MMA issuers run their loops with the whole warp and
+// predicate the instructions themselves (`lead`, below): behind a branch of one lane every operand is
+// moved to a uniform register anew: 60 clocks per MMA, 640 per k-block of 4 MMAs, 2 commits and 2 waits,
+// where a 128-token tile needs 256 of the tensor core; so 450 (d 768, 4 layers, 120 tokens: 182 -> 167 us a
+// forward, 10 tokens 147 -> 134; d 2048, 2 layers, 120 tokens 139 -> 127; 4 layers of d 4096, 120 tokens 421 ->
+// 415, 512 tokens 839 -> 820).
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e;
+}
+
+// The four MMAs of a 64-wide k-block (descriptors 32 bytes apart), by the thread with `lead`.  accumulate = 0:
+// the first one overwrites D.
+template <int CG = 1>
+__device__ __forceinline__ void tc_mma_kblock(uint32_t lead, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                              uint32_t idesc, uint32_t accumulate) {
+  if constexpr (CG == 1)
+    asm volatile(
+        "{\n .reg .pred e, p, t;\n .reg .b64 a1, b1, a2, b2, a3, b3;\n"
+        " setp.ne.b32 e, %5, 0;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, 0, 0;\n"
+        " add.s64 a1, %1, 2;\n add.s64 b1, %2, 2;\n add.s64 a2, %1, 4;\n add.s64 b2, %2, 4;\n"
+        " add.s64 a3, %1, 6;\n add.s64 b3, %2, 6;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, t;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, t;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, t;\n}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
+        : "memory");
+  else
+    asm volatile(
+        "{\n .reg .pred e, p, t;\n .reg .b64 a1, b1, a2, b2, a3, b3;\n"
+        " setp.ne.b32 e, %5, 0;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, 0, 0;\n"
+        " add.s64 a1, %1, 2;\n add.s64 b1, %2, 2;\n add.s64 a2, %1, 4;\n add.s64 b2, %2, 4;\n"
+        " add.s64 a3, %1, 6;\n add.s64 b3, %2, 6;\n"
+        " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
+        " @e tcgen05.mma.cta_group::2.kind::f16 [%0], a1, b1, %3, t;\n"
+        " @e tcgen05.mma.cta_group::2.kind::f16 [%0], a2, b2, %3, t;\n"
+        " @e tcgen05.mma.cta_group::2.kind::f16 [%0], a3, b3, %3, t;\n}" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
+        : "memory");
+}
+
+// tc_commit, expect_tx and TMA loads by the thread with `lead`
+template <int CG = 1>
+__device__ __forceinline__ void tc_commit_lead(uint32_t lead, uint64_t* bar, uint16_t pair = 3) {
+  if constexpr (CG == 1)
+    asm volatile(
+        "{\n .reg .pred e;\n setp.ne.b32 e, %1, 0;\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(smem_u32(bar)),
+        "r"(lead)
+        : "memory");
+  else
+    asm volatile(
+        "{\n .reg .pred e;\n setp.ne.b32 e, %2, 0;\n"
+        " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}" ::"r"(
+            smem_u32(bar)),
+        "h"(pair), "r"(lead)
+        : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx_lead(uint32_t lead, uint64_t* bar, uint32_t bytes) {
+  asm volatile("{\n .reg .pred e;\n setp.ne.b32 e, %2, 0;\n @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(
+                   smem_u32(bar)),
+               "r"(bytes), "r"(lead)
+               : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_lead(uint32_t lead, void* smem_dst, const CUtensorMap* map, uint64_t* bar,
+                                                 int x, int y, uint64_t policy) {
+  asm volatile(
+      "{\n .reg .pred e;\n setp.ne.b32 e, %6, 0;\n"
+      " @e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3}], [%4], %5;\n}" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(policy), "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_lead(uint32_t lead, void* smem_dst, const CUtensorMap* map, uint64_t* bar,
+                                                 int x, int y, int z, uint64_t policy) {
+  asm volatile(
+      "{\n .reg .pred e;\n setp.ne.b32 e, %7, 0;\n"
+      " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3, %4}], [%5], %6;\n}" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(policy), "r"(lead)
+      : "memory");
+}
+
 // Shared-memory matrix descriptor for a K-major operand tile written by TMA with 128-byte
 // swizzle: rows of 128 bytes (64 bf16), 8-row atoms of 1024 bytes stacked contiguously.
 //   bits  0-13 start address >> 4; bits 16-29 leading byte offset >> 4 (unused for this layout);

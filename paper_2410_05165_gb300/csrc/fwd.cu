@@ -146,12 +146,12 @@ __device__ __forceinline__ GP gemm_phase(const FwdParams& p, int gi, int BN) {
 
 // Copy of one stage of weight tile mt: 128 rows x 64 k, one box (SwiGLU: 64 gate rows and the
 // matching 64 up rows of a three-dimensional map [gate | up][d_ffn][d]).
-__device__ __forceinline__ void load_weights(const GP& g, const CUtensorMap* map, uint8_t* dst, uint64_t* bar, int mt,
-                                             int kx, uint64_t pol) {
+__device__ __forceinline__ void load_weights(uint32_t lead, const GP& g, const CUtensorMap* map, uint8_t* dst,
+                                             uint64_t* bar, int mt, int kx, uint64_t pol) {
   if (g.epi == EPI_SWIGLU)
-    tma_load_3d_cg<1>(dst, map, smem_u32(bar), kx, mt * 64, 0, pol);
+    tma_load_3d_lead(lead, dst, map, bar, kx, mt * 64, 0, pol);
   else
-    tma_load_2d(dst, map, bar, kx, mt * GEMM_BM, pol);
+    tma_load_2d_lead(lead, dst, map, bar, kx, mt * GEMM_BM, pol);
 }
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* a) {
@@ -249,6 +249,10 @@ __device__ bool mwait(uint64_t* bar, uint32_t parity, unsigned* err) {
       }
     }
   }
+}
+// the same by every lane of a converged warp
+__device__ __forceinline__ bool mwait_warp(uint64_t* bar, uint32_t parity, unsigned* err) {
+  return __all_sync(0xffffffffu, mwait(bar, parity, err));
 }
 
 // trs: the n-tile's norm scales (QKV / gate-up).  (The residual updates of the O / down projections have
@@ -708,7 +712,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsRoles));
   if (warp == 0) {
     // ------------------------------------------------------------- weight producer (never waits for the grid)
-    if (lane == 0) {
+    {   // (the whole warp, one thread elected, as in the two roles below)
+      const uint32_t lead = elect_one();
       const uint64_t pol = policy_evict_first();
       int s = 0;
       uint32_t ph = 0;
@@ -722,13 +727,13 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
         while (ok && it.next(g.w, tile, k0, k1)) {
           const int mt = tile / g.n_tiles;
           for (int kbi = k0; kbi < k1; ++kbi) {
-            if (!mwait(&emptyA[s], ph ^ 1u, p.err)) {
+            if (!mwait_warp(&emptyA[s], ph ^ 1u, p.err)) {
               ok = false;
               break;
             }
-            mbar_arrive_expect_tx(&fullA[s], C::A_BYTES);
+            mbar_expect_tx_lead(lead, &fullA[s], C::A_BYTES);
             lastA[s] = (int)ph;
-            load_weights(g, mA, ringA + s * C::A_BYTES, &fullA[s], mt, kbi * GEMM_BK, pol);
+            load_weights(lead, g, mA, ringA + s * C::A_BYTES, &fullA[s], mt, kbi * GEMM_BK, pol);
             if (++s == C::SA) {
               s = 0;
               ph ^= 1u;
@@ -740,7 +745,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------- activation producer
-    if (lane == 0) {
+    {
+      const uint32_t lead = elect_one();
       const uint64_t pol = policy_evict_last();
       int s = 0;
       uint32_t ph = 0;
@@ -750,12 +756,12 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
         const int nu = cta_units(g.w, c);
         // the compute warps pass the grid barrier that publishes this phase's input and count it in
         // `go` (one grid poller per CTA)
-        if (!cta_count_wait(go, gi + 1, p.err)) {
+        if (!__all_sync(0xffffffffu, cta_count_wait(go, gi + 1, p.err))) {
           ok = false;
           break;
         }
         if (nu == 0) continue;
-        if (p.trace) p.trace[((size_t)1 * (7 * L + 2) + gi) * G + c] = globaltimer_ns();
+        if (p.trace && lane == 0) p.trace[((size_t)1 * (7 * L + 2) + gi) * G + c] = globaltimer_ns();
         fence_proxy_async();
         const CUtensorMap* mB = p.maps + g.mapB;
         SegIter it;
@@ -764,26 +770,27 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
         while (ok && it.next(g.w, tile, k0, k1)) {
           const int nt = tile % g.n_tiles;
           for (int kbi = k0; kbi < k1; ++kbi) {
-            if (!mwait(&emptyB[s], ph ^ 1u, p.err)) {
+            if (!mwait_warp(&emptyB[s], ph ^ 1u, p.err)) {
               ok = false;
               break;
             }
-            mbar_arrive_expect_tx(&fullB[s], C::B_BYTES);
+            mbar_expect_tx_lead(lead, &fullB[s], C::B_BYTES);
             lastB[s] = (int)ph;
-            tma_load_2d(ringB + s * C::B_BYTES, mB, &fullB[s], kbi * GEMM_BK, nt * BN, pol);
+            tma_load_2d_lead(lead, ringB + s * C::B_BYTES, mB, &fullB[s], kbi * GEMM_BK, nt * BN, pol);
             if (++s == C::SB) {
               s = 0;
               ph ^= 1u;
             }
           }
         }
-        if (p.trace) p.trace[((size_t)2 * (7 * L + 2) + gi) * G + c] = globaltimer_ns();
+        if (p.trace && lane == 0) p.trace[((size_t)2 * (7 * L + 2) + gi) * G + c] = globaltimer_ns();
       }
       if (!ok) *failed = 1;
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    {
+      const uint32_t lead = elect_one();
       constexpr uint32_t idesc = idesc_bf16_f32(GEMM_BM, BN);
       int sa = 0, sb = 0;
       uint32_t pa = 0, pb = 0;
@@ -801,25 +808,23 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
           const int len = k1 - k0;
           const int acc = si & 1, use = si >> 1;
           ++si;
-          if (!mwait(&tempty[acc], (uint32_t)(use & 1) ^ 1u, p.err)) {
+          if (!mwait_warp(&tempty[acc], (uint32_t)(use & 1) ^ 1u, p.err)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t dt = tmem_base + (uint32_t)(acc * BN);
           for (int j = 0; j < len; ++j) {
-            if (!mwait(&fullA[sa], pa, p.err) || !mwait(&fullB[sb], pb, p.err)) {
+            if (!__all_sync(0xffffffffu, mwait(&fullA[sa], pa, p.err) && mwait(&fullB[sb], pb, p.err))) {
               ok = false;
               break;
             }
             tc_fence_after();
             const uint64_t ad = smem_desc_sw128(smem_u32(ringA + sa * C::A_BYTES));
             const uint64_t bd = smem_desc_sw128(smem_u32(ringB + sb * C::B_BYTES));
-#pragma unroll
-            for (int kk = 0; kk < GEMM_BK / 16; ++kk)
-              tc_mma_bf16(dt, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc, (j > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(&emptyA[sa]);
-            tc_commit(&emptyB[sb]);
+            tc_mma_kblock(lead, dt, ad, bd, idesc, j > 0 ? 1u : 0u);
+            tc_commit_lead(lead, &emptyA[sa]);
+            tc_commit_lead(lead, &emptyB[sb]);
             if (++sa == C::SA) {
               sa = 0;
               pa ^= 1u;
@@ -830,18 +835,18 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
             }
           }
           if (!ok) break;
-          tc_commit(&tfull[acc]);
+          tc_commit_lead(lead, &tfull[acc]);
         }
-        if (p.trace && any) {
+        if (p.trace && any) {   // (every lane waits)
           // time the last MMA of this phase completed
-          tc_commit(mma_done);
+          tc_commit_lead(lead, mma_done);
           mbar_wait(mma_done, (uint32_t)(mma_waits & 1), nullptr);
           ++mma_waits;
-          p.trace[((size_t)3 * (7 * L + 2) + gi) * G + c] = globaltimer_ns();
+          if (lane == 0) p.trace[((size_t)3 * (7 * L + 2) + gi) * G + c] = globaltimer_ns();
         }
       }
       if (!ok) *failed = 1;
-      tc_commit(mma_done);
+      tc_commit_lead(lead, mma_done);
       mbar_wait(mma_done, (uint32_t)(mma_waits & 1), nullptr);
     }
   }
