@@ -112,38 +112,42 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
       : "memory");
 }
 
-// tma_load_2d / tma_load_3d into this CTA's shared memory whose bytes an mbarrier of either CTA of a
-// pair counts (CG = 2, `bar` a cluster address), or this CTA's (CG = 1).
+// Loads by the thread with `lead` (elect_one, below) into this CTA's shared memory whose bytes an mbarrier of
+// either CTA of a pair counts (CG = 2, `bar` a cluster address), or this CTA's (CG = 1).
 template <int CG>
-__device__ __forceinline__ void tma_load_2d_cg(void* smem_dst, const CUtensorMap* map, uint32_t bar, int x, int y,
-                                               uint64_t policy) {
+__device__ __forceinline__ void tma_load_2d_cg(uint32_t lead, void* smem_dst, const CUtensorMap* map, uint32_t bar,
+                                               int x, int y, uint64_t policy) {
   if constexpr (CG == 1)
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-        " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(smem_dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "l"(policy)
+        "{\n .reg .pred e;\n setp.ne.b32 e, %6, 0;\n"
+        " @e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3}], [%4], %5;\n}" ::"r"(smem_u32(smem_dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "l"(policy), "r"(lead)
         : "memory");
   else
     asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-        " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(smem_dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "l"(policy)
+        "{\n .reg .pred e;\n setp.ne.b32 e, %6, 0;\n"
+        " @e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3}], [%4], %5;\n}" ::"r"(smem_u32(smem_dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "l"(policy), "r"(lead)
         : "memory");
 }
 template <int CG>
-__device__ __forceinline__ void tma_load_3d_cg(void* smem_dst, const CUtensorMap* map, uint32_t bar, int x, int y,
-                                               int z, uint64_t policy) {
+__device__ __forceinline__ void tma_load_3d_cg(uint32_t lead, void* smem_dst, const CUtensorMap* map, uint32_t bar,
+                                               int x, int y, int z, uint64_t policy) {
   if constexpr (CG == 1)
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-        " [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(smem_u32(smem_dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy)
+        "{\n .reg .pred e;\n setp.ne.b32 e, %7, 0;\n"
+        " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3, %4}], [%5], %6;\n}" ::"r"(smem_u32(smem_dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy), "r"(lead)
         : "memory");
   else
     asm volatile(
-        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-        " [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(smem_u32(smem_dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy)
+        "{\n .reg .pred e;\n setp.ne.b32 e, %7, 0;\n"
+        " @e cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3, %4}], [%5], %6;\n}" ::"r"(smem_u32(smem_dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy), "r"(lead)
         : "memory");
 }
 
@@ -217,39 +221,20 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, bf16 inputs, fp32 accumulate.  CG = 2 (M = 256): A rows and D lanes
-// 0-127 are CTA 0's, 128-255 CTA 1's; the first half of B's rows is read from CTA 0's shared memory
-// and the second from CTA 1's (the same offsets in both); D has all N columns in both CTAs' TMEM.
-template <int CG = 1>
+// D[tmem] (+)= A[smem] * B[smem]^T, bf16 inputs, fp32 accumulate (one thread).
 __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                             uint32_t accumulate) {
-  if constexpr (CG == 1)
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-  else
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
 }
 
-// Arrive on an mbarrier (CG = 2: at this offset in both CTAs, the cluster ranks of `pair`) once every
-// previously issued tcgen05.mma of this thread has completed.
-template <int CG = 1>
-__device__ __forceinline__ void tc_commit(uint64_t* bar, uint16_t pair = 3) {
-  if constexpr (CG == 1)
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-  else
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            smem_u32(bar)),
-        "h"(pair)
-        : "memory");
+// Arrive on an mbarrier once every previously issued tcgen05.mma of this thread has completed.
+__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+               : "memory");
 }
 
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp gets lane (base + i), 32 values.
@@ -287,7 +272,9 @@ __device__ __forceinline__ uint32_t elect_one() {
 }
 
 // The four MMAs of a 64-wide k-block (descriptors 32 bytes apart), by the thread with `lead`.  accumulate = 0:
-// the first one overwrites D.
+// the first one overwrites D.  CG = 2 (M = 256): A rows and D lanes 0-127 are CTA 0's, 128-255 CTA 1's; the
+// first half of B's rows is read from CTA 0's shared memory and the second from CTA 1's (the same offsets in
+// both); D has all N columns in both CTAs' TMEM.
 template <int CG = 1>
 __device__ __forceinline__ void tc_mma_kblock(uint32_t lead, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                               uint32_t idesc, uint32_t accumulate) {
@@ -317,7 +304,8 @@ __device__ __forceinline__ void tc_mma_kblock(uint32_t lead, uint32_t d_tmem, ui
         : "memory");
 }
 
-// tc_commit, expect_tx and TMA loads by the thread with `lead`
+// tc_commit (CG = 2: at this offset in both CTAs, the cluster ranks of `pair`) and expect_tx by the thread
+// with `lead`
 template <int CG = 1>
 __device__ __forceinline__ void tc_commit_lead(uint32_t lead, uint64_t* bar, uint16_t pair = 3) {
   if constexpr (CG == 1)
@@ -340,25 +328,6 @@ __device__ __forceinline__ void mbar_expect_tx_lead(uint32_t lead, uint64_t* bar
                "r"(bytes), "r"(lead)
                : "memory");
 }
-__device__ __forceinline__ void tma_load_2d_lead(uint32_t lead, void* smem_dst, const CUtensorMap* map, uint64_t* bar,
-                                                 int x, int y, uint64_t policy) {
-  asm volatile(
-      "{\n .reg .pred e;\n setp.ne.b32 e, %6, 0;\n"
-      " @e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%2, %3}], [%4], %5;\n}" ::"r"(smem_u32(smem_dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(policy), "r"(lead)
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_3d_lead(uint32_t lead, void* smem_dst, const CUtensorMap* map, uint64_t* bar,
-                                                 int x, int y, int z, uint64_t policy) {
-  asm volatile(
-      "{\n .reg .pred e;\n setp.ne.b32 e, %7, 0;\n"
-      " @e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%2, %3, %4}], [%5], %6;\n}" ::"r"(smem_u32(smem_dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(policy), "r"(lead)
-      : "memory");
-}
-
 // Shared-memory matrix descriptor for a K-major operand tile written by TMA with 128-byte
 // swizzle: rows of 128 bytes (64 bf16), 8-row atoms of 1024 bytes stacked contiguously.
 //   bits  0-13 start address >> 4; bits 16-29 leading byte offset >> 4 (unused for this layout);

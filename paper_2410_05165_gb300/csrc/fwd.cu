@@ -149,9 +149,9 @@ __device__ __forceinline__ GP gemm_phase(const FwdParams& p, int gi, int BN) {
 __device__ __forceinline__ void load_weights(uint32_t lead, const GP& g, const CUtensorMap* map, uint8_t* dst,
                                              uint64_t* bar, int mt, int kx, uint64_t pol) {
   if (g.epi == EPI_SWIGLU)
-    tma_load_3d_lead(lead, dst, map, bar, kx, mt * 64, 0, pol);
+    tma_load_3d_cg<1>(lead, dst, map, smem_u32(bar), kx, mt * 64, 0, pol);
   else
-    tma_load_2d_lead(lead, dst, map, bar, kx, mt * GEMM_BM, pol);
+    tma_load_2d_cg<1>(lead, dst, map, smem_u32(bar), kx, mt * GEMM_BM, pol);
 }
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* a) {
@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
             }
             mbar_expect_tx_lead(lead, &fullB[s], C::B_BYTES);
             lastB[s] = (int)ph;
-            tma_load_2d_lead(lead, ringB + s * C::B_BYTES, mB, &fullB[s], kbi * GEMM_BK, nt * BN, pol);
+            tma_load_2d_cg<1>(lead, ringB + s * C::B_BYTES, mB, smem_u32(&fullB[s]), kbi * GEMM_BK, nt * BN, pol);
             if (++s == C::SB) {
               s = 0;
               ph ^= 1u;

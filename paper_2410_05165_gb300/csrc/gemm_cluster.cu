@@ -28,10 +28,11 @@
 // 53.1 -> 46.2; 128: [19456 x 4096] x 120 29.9 -> 28.6).
 //
 // Measured against the stream-K kernel / two narrow CTAs per SM (us, GB300): [12288 x 4096] x 120 tokens
-// 32.1 / 23.7 -> 22.7 (4.5 TB/s), x 200 31.4 -> 24.6 (narrow), x 10 20.1 -> 21.4 (narrow; the one loss: an SM
-// takes in 60 bytes per ns, and 96 of 152 are used), [4096 x 11008] x 120 31.4 / 24.7 -> 20.6, x 200 35.6
-// -> 25.7 (narrow), [4096 x 4096] x 120 23.3 / 16.2 -> 12.4, [768 x 768] x 10 9.4 / 6.5 -> 5.8, [4096 x 11008] x
-// 512 56.6 / 46.3 -> 34.4, x 960 90.2 / 72.6 -> 55.3.
+// 32.1 / 23.7 -> 20.2 (5.0 TB/s), x 200 31.4 -> 25.1 (narrow), x 10 20.1 -> 18.8 (narrow),
+// [4096 x 11008] x 120 31.4 / 24.7 -> 19.8, x 200 35.6 -> 25.3 (narrow), [4096 x 4096] x 120 23.3 / 16.2 -> 11.7,
+// [768 x 768] x 10 9.4 / 6.5 -> 5.6, [4096 x 11008] x 512 56.6 / 46.3 -> 34.8, x 960 90.2 / 72.6 -> 56.2.
+// Of these the converged producer and issuer (elect_one) gave 22.9 -> 20.2, 21.3 -> 18.8, 20.6 -> 19.8, 12.4 -> 11.7;
+// [256 x 11008] x 10 12.1 -> 9.7.
 // Error against fp64 (relative, stream-K kernel / here): [4096 x 11008] 2.3e-6 / 1.4e-6, [4096 x 4096] 7.9e-7 /
 // 4.7e-7, [768 x 768] 0.9e-7 / 1.1e-7, [22016 x 4096] 4.2e-6 / 4.4e-6.
 //
@@ -149,8 +150,9 @@ __global__ void __launch_bounds__(THREADS, 2)
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------------------------ TMA producer
+    {
+      // ------------------------------------------------------------------ TMA producer (converged, one elected thread)
+      const uint32_t lead_t = elect_one();
       // weights read by one token tile alone are streamed past the cache
       const uint64_t pol_w = p.n_tiles == 1 ? policy_evict_first() : policy_evict_last();
       const uint64_t pol_x = policy_evict_last();
@@ -165,17 +167,17 @@ __global__ void __launch_bounds__(THREADS, 2)
       int stage = 0;
       uint32_t phase = 0;
       for (int k = k0; k < k1; ++k) {
-        if (!mbar_wait(&empty[stage], phase ^ 1u, p.err)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&empty[stage], phase ^ 1u, p.err))) {
           *failed = 1;
           break;
         }
         uint8_t* sa = smem + stage * C::STAGE_BYTES;
         // (a pair's copies all count on the issuing CTA's barrier)
         const uint32_t fb = CG == 2 ? mapa_u32(&full[stage], (uint32_t)lead) : smem_u32(&full[stage]);
-        if (half == 0) mbar_arrive_expect_tx(&full[stage], CG * C::STAGE_BYTES);
-        tma_load_2d_cg<CG>(sa, &tmA, fb, k * GEMM_BK, r0, pol_w);
-        tma_load_2d_cg<CG>(sa + 8192, &tmA, fb, k * GEMM_BK, r1, pol_w);
-        tma_load_2d_cg<CG>(sa + C::A_BYTES, &tmB, fb, k * GEMM_BK, n_tile * BN + half * (BN / CG), pol_x);
+        if (half == 0) mbar_expect_tx_lead(lead_t, &full[stage], CG * C::STAGE_BYTES);
+        tma_load_2d_cg<CG>(lead_t, sa, &tmA, fb, k * GEMM_BK, r0, pol_w);
+        tma_load_2d_cg<CG>(lead_t, sa + 8192, &tmA, fb, k * GEMM_BK, r1, pol_w);
+        tma_load_2d_cg<CG>(lead_t, sa + C::A_BYTES, &tmB, fb, k * GEMM_BK, n_tile * BN + half * (BN / CG), pol_x);
         if (++stage == stages) {
           stage = 0;
           phase ^= 1u;
@@ -183,31 +185,29 @@ __global__ void __launch_bounds__(THREADS, 2)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && half == 0) {
-      // ------------------------------------------------------------------ MMA issuer
+    if (half == 0) {
+      // ------------------------------------------------------------------ MMA issuer (converged, one elected thread)
+      const uint32_t lead_t = elect_one();
       constexpr uint32_t idesc = idesc_bf16_f32(CG * GEMM_BM, BN);
       const uint16_t pair = (uint16_t)(3u << lead);
       int stage = 0;
       uint32_t phase = 0;
       for (int k = k0; k < k1; ++k) {
-        if (!mbar_wait(&full[stage], phase, p.err)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&full[stage], phase, p.err))) {
           *failed = 1;
           break;
         }
         tc_fence_after();
         const uint32_t sa = smem_u32(smem + stage * C::STAGE_BYTES);
         const uint64_t ad = smem_desc_sw128(sa), bd = smem_desc_sw128(sa + C::A_BYTES);
-#pragma unroll
-        for (int kk = 0; kk < GEMM_BK / 16; ++kk)
-          tc_mma_bf16<CG>(k < k2 ? tmem_base : tmem_base + BN, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc,
-                      ((k != k0 && k != k2) || kk > 0) ? 1u : 0u);
-        tc_commit<CG>(&empty[stage], pair);
+        tc_mma_kblock<CG>(lead_t, k < k2 ? tmem_base : tmem_base + BN, ad, bd, idesc, k != k0 && k != k2 ? 1u : 0u);
+        tc_commit_lead<CG>(lead_t, &empty[stage], pair);
         if (++stage == stages) {
           stage = 0;
           phase ^= 1u;
         }
       }
-      tc_commit<CG>(tfull, pair);   // (also after a failure: nothing may run when TMEM is released)
+      tc_commit_lead<CG>(lead_t, tfull, pair);   // (also after a failure: nothing may run when TMEM is released)
     }
   }
   __syncwarp();   // (the other lanes of the role warps do not poll beside their lane 0)

@@ -9,7 +9,8 @@
 // remainder (WorkSplit over pairs, gemm_core.cuh); split tiles are summed by the last pair to publish,
 // each CTA its 128 rows, in k order, while the whole tiles' MMAs run.  No CTA waits for another pair.
 //
-// Measured (GB300, us, one-CTA stream-K kernel / this one): [22016 x 4096] x 3840 tokens 419 / 369
+// Measured (GB300, us, one-CTA stream-K kernel / this one; a slower box, 395 -> 375 with the converged producer
+// and issuer of elect_one, is not counted): [22016 x 4096] x 3840 tokens 419 / 369
 // (1.88 PFLOP/s), [19456 x 4096] x 1024 tokens 113 / 94, x 1024 (K) x 3840 tokens 141 / 112.
 //
 // Roles (320 threads): warp 0 = TMA producer, warp 1 = TMEM + MMA issue (CTA 0's issues for both), warps
@@ -91,8 +92,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------------------------ TMA producer
+    {
+      // ------------------------------------------------------------------ TMA producer (converged, one elected thread)
+      const uint32_t lead_t = elect_one();
       tma_prefetch_desc(&tmA);
       tma_prefetch_desc(&tmB);
       const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
@@ -105,19 +107,19 @@ __global__ void __launch_bounds__(THREADS, 1)
       while (ok && it.next(p.w, tile, k0, k1)) {
         const int mt = 2 * (tile / p.n_tiles) + rank, brow = tile % p.n_tiles * BN + rank * (BN / 2);
         for (int k = k0; k < k1; ++k) {
-          if (!mbar_wait(&empty[stage], phase ^ 1u, p.err)) {
+          if (!__all_sync(0xffffffffu, mbar_wait(&empty[stage], phase ^ 1u, p.err))) {
             ok = false;
             break;
           }
           uint8_t* sa = smem + stage * STAGE_BYTES;
           const uint32_t fb = mapa_u32(&full[stage], 0);
-          if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * STAGE_BYTES);
+          if (rank == 0) mbar_expect_tx_lead(lead_t, &full[stage], 2 * STAGE_BYTES);
           last_fill[stage] = (int)phase;
           if constexpr (EPI == EPI_SWIGLU)   // 64 gate rows and the matching 64 up rows
-            tma_load_3d_cg<2>(sa, &tmA, fb, k * GEMM_BK, mt * 64, 0, pol_w);
+            tma_load_3d_cg<2>(lead_t, sa, &tmA, fb, k * GEMM_BK, mt * 64, 0, pol_w);
           else
-            tma_load_2d_cg<2>(sa, &tmA, fb, k * GEMM_BK, mt * GEMM_BM, pol_w);
-          tma_load_2d_cg<2>(sa + A_BYTES, &tmB, fb, k * GEMM_BK, brow, pol_x);
+            tma_load_2d_cg<2>(lead_t, sa, &tmA, fb, k * GEMM_BK, mt * GEMM_BM, pol_w);
+          tma_load_2d_cg<2>(lead_t, sa + A_BYTES, &tmB, fb, k * GEMM_BK, brow, pol_x);
           if (++stage == STAGES) {
             stage = 0;
             phase ^= 1u;
@@ -127,8 +129,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (!ok) *failed = 1;
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      // ------------------------------------------------------------------ MMA issuer
+    if (rank == 0) {
+      // ------------------------------------------------------------------ MMA issuer (converged, one elected thread)
+      const uint32_t lead_t = elect_one();
       constexpr uint32_t idesc = idesc_bf16_f32(2 * GEMM_BM, BN);
       int stage = 0, si = 0;
       uint32_t phase = 0;
@@ -138,35 +141,33 @@ __global__ void __launch_bounds__(THREADS, 1)
       int tile, k0, k1;
       for (; ok && it.next(p.w, tile, k0, k1); ++si) {
         const int acc = si & 1, use = si >> 1;
-        if (!mbar_wait(&tempty[acc], (uint32_t)(use & 1) ^ 1u, p.err)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&tempty[acc], (uint32_t)(use & 1) ^ 1u, p.err))) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t dt = tmem_base + (uint32_t)(acc * BN);
         for (int k = k0; k < k1; ++k) {
-          if (!mbar_wait(&full[stage], phase, p.err)) {
+          if (!__all_sync(0xffffffffu, mbar_wait(&full[stage], phase, p.err))) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + stage * STAGE_BYTES);
           const uint64_t ad = smem_desc_sw128(sa), bd = smem_desc_sw128(sa + A_BYTES);
-#pragma unroll
-          for (int kk = 0; kk < GEMM_BK / 16; ++kk)
-            tc_mma_bf16<2>(dt, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc, (k > k0 || kk > 0) ? 1u : 0u);
-          tc_commit<2>(&empty[stage]);
+          tc_mma_kblock<2>(lead_t, dt, ad, bd, idesc, k > k0 ? 1u : 0u);
+          tc_commit_lead<2>(lead_t, &empty[stage]);
           if (++stage == STAGES) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        tc_commit<2>(&tfull[acc]);
+        tc_commit_lead<2>(lead_t, &tfull[acc]);
       }
       if (!ok) *failed = 1;
       // no MMA may still be running when TMEM is released: both CTAs wait for this commit at the end
-      tc_commit<2>(mma_done);
+      tc_commit_lead<2>(lead_t, mma_done);
     }
   } else {
     // -------------------------------------------------------------------- epilogue
