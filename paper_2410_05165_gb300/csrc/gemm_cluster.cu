@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(THREADS, 2)
       tc_commit_lead<CG>(lead_t, tfull, pair);   // (also after a failure: nothing may run when TMEM is released)
     }
   }
-  __syncwarp();   // (the other lanes of the role warps do not poll beside their lane 0)
+  __syncwarp();
   // Every thread waits for the accumulator: all of this CTA's MMAs are done, so all of its ring's
   // copies have landed and been read (after a failure: those of the stages that were consumed).
   if (!mbar_wait(tfull, 0, p.err)) *failed = 1;

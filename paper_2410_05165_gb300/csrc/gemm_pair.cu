@@ -10,7 +10,8 @@
 // each CTA its 128 rows, in k order, while the whole tiles' MMAs run.  No CTA waits for another pair.
 //
 // Measured (GB300, us, one-CTA stream-K kernel / this one): [22016 x 4096] x 3840 tokens 419 / 369, and 355
-// (1.95 PFLOP/s, tensor pipe 91% active) with the converged producer and issuer (elect_one), [19456 x 4096] x 1024 tokens 113 / 94, x 1024 (K) x 3840 tokens 141 / 112.
+// (1.95 PFLOP/s, tensor pipe 91% active) with the converged producer and issuer (elect_one);
+// [19456 x 4096] x 1024 tokens 113 / 94, x 1024 (K) x 3840 tokens 141 / 112.
 //
 // Roles (320 threads): warp 0 = TMA producer, warp 1 = TMEM + MMA issue (CTA 0's issues for both), warps
 // 2-9 = two epilogue warpgroups (TMEM lane quadrant = warp % 4), alternate 32-token chunks each.
