@@ -184,6 +184,11 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
       ldsm_x4(qbase + (uint32_t)((r * HD + q_chunk<HD>(r, kk * 2 + cofs) * 8) * 2), qf[kk][0], qf[kk][1], qf[kk][2],
               qf[kk][3]);
   }
+  // The vote at the first step lets thread 0 copy K/V over the Q tile.  A barrier alone does not order the
+  // fragment loads before that copy (another proxy): without the fence a warp that ran late had K/V rows for Q
+  // (heads of 32, many CTAs per SM).  The same goes for the K/V fragments of each step, below.  (Both fences
+  // together: operator kernels +1.4% on average, no change of a forward.)
+  fence_proxy_async_shared();
   const int g = lane >> 2, tq = lane & 3;
   const int row_a = warp * 16 + g, row_b = row_a + 8;
   const int vis_a = row_a < nq ? a.tok_vis[t0 + row_a] : 0;
@@ -326,6 +331,7 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
         }
       }
     }
+    fence_proxy_async_shared();   // (the next step's vote hands this buffer to a copy)
     if (++buf == D) buf = 0;
     if (st < 2) ATT_TR(3 + 2 * st);
   }

@@ -151,6 +151,14 @@ __device__ __forceinline__ void tma_load_3d_cg(uint32_t lead, void* smem_dst, co
         : "memory");
 }
 
+// Orders this thread's own (generic-proxy) accesses with TMA copies (the async proxy) of the same addresses:
+// its stores before copies that read them, its loads and stores before copies that overwrite them.  Followed
+// by whatever tells the copying thread.  (_global, _shared: of that memory alone; _global also after a wait,
+// before copies that read what others stored.)
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+__device__ __forceinline__ void fence_proxy_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------------------------
 // thread-block clusters
 // ---------------------------------------------------------------------------------------------

@@ -170,7 +170,6 @@ __device__ __forceinline__ int atom_acq_rel_add(int* a, int v) {
   asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(a), "r"(v) : "memory");
   return old;
 }
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 __device__ __forceinline__ bool err_set(const unsigned* e) { return *(volatile const unsigned*)e != 0u; }
 
@@ -762,7 +761,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
         }
         if (nu == 0) continue;
         if (p.trace && lane == 0) p.trace[((size_t)1 * (7 * L + 2) + gi) * G + c] = globaltimer_ns();
-        fence_proxy_async();
+        fence_proxy_async_global();
         const CUtensorMap* mB = p.maps + g.mapB;
         SegIter it;
         it.init(g.w, c);
@@ -899,7 +898,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
           ok = false;
           break;
         }
-        fence_proxy_async();
+        fence_proxy_async_global();
         named_bar_sync(1, CT);
       }
       if (kind == 0 || kind == 4) {
@@ -920,7 +919,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) fwd_kernel(const FwdParams p) 
       }
       if (p.trace && ctid == 0) p.trace[(size_t)ph * G + c] = globaltimer_ns();
       // publish this phase: this CTA's generic-proxy stores must be visible to the other CTAs'
-      // TMA (async-proxy) reads of the next phases, hence the proxy fence before the release
+      // TMA (async-proxy) reads of the next phases, and its accesses to staging buffers and tables come
+      // before the next phases' copies into that shared memory, hence the proxy fence before the release
       if (ph < NP - 1) {
         fence_proxy_async();
         __threadfence();

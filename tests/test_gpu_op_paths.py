@@ -97,7 +97,10 @@ def test_rmsnorm_paths(ats, T, d, pad):
                                             (5, 64, 128, 63, False), (32, 128, 200, 330, True), (40, 32, 300, 250, True),
                                             (32, 64, 130, 650, True), (32, 128, 321, 641, False), (2, 32, 0, 5, True),
                                             (1, 128, 2100, 64, True), (80, 32, 70, 257, False), (2, 32, 70, 1300, True),
-                                            (3, 64, 200, 7700, False), (12, 64, 1000, 1000, False), (4, 32, 1000, 700, False)])
+                                            (3, 64, 200, 7700, False), (12, 64, 1000, 1000, False), (4, 32, 1000, 700, False),
+                                            # (many CTAs per SM: warps that run late still read their own Q and K/V tiles)
+                                            (120, 32, 128, 256, True), (32, 32, 300, 1024, True), (120, 64, 500, 256, True),
+                                            (120, 32, 200, 256, False), (32, 32, 1000, 1000, False)])
 def test_attention_paths(ats, H, hd, P, T, paths):
     rng = np.random.default_rng(H + P + T)
     d, n = H * hd, (P + 63) // 64
