@@ -87,8 +87,8 @@ struct AttCfg {
 // (count 1); par: bit b is the parity of buffer b's next fill (zero at first), kept identically by
 // every thread from item to item.  Writes the normalised output (a.direct) or the split's
 // unnormalised partials.  Returns false if a bounded wait timed out.
-// Sink::kCustom: the split's share of the tile's visible pages is balanced over user_splits, and the
-// partials go to sink(o, m, l of the thread's two rows) instead (both known at compile time).
+// Sink::kCustom: the partials go to sink(o, m, l of the thread's two rows) instead, and with chunks_per_split = 0
+// the tile's visible pages are balanced over user_splits.
 // D - 1 copies are in flight ahead of the arithmetic: a step of 32 keys takes ~0.5 us of tensor and
 // softmax work, a copy 1.5 - 2 us (more from DRAM), so two buffers left the warps waiting for copies.
 struct AttGlobalSink {
@@ -118,12 +118,12 @@ __device__ bool attn_item(const AttnArgs& a, const CUtensorMap* mk, const CUtens
   constexpr int BOXW = HD >= 64 ? 64 : HD;
   const int nch = (a.qt_vis[tile] + ATT_PAGE - 1) / ATT_PAGE;
   int c0 = 0, c1 = nch;
-  if constexpr (Sink::kCustom) {
-    c0 = split * nch / S_u;
-    c1 = (split + 1) * nch / S_u;
-  } else if (a.chunks_per_split > 0) {
+  if (a.chunks_per_split > 0) {
     c0 = min(nch, split * a.chunks_per_split);
     c1 = min(nch, c0 + a.chunks_per_split);
+  } else if constexpr (Sink::kCustom) {
+    c0 = split * nch / S_u;
+    c1 = (split + 1) * nch / S_u;
   }
   ATT_TR(0);
   constexpr int SUBS = ATT_PAGE / ATT_SUB;

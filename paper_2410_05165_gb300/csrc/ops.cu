@@ -54,17 +54,35 @@ atspeed_status run_gemm(cudaStream_t st, const GemmArgs& a, void* ws) {
   return gemm_status(gemm_pair_launch(a, s, grid, st, eb, sizeof eb));
 }
 
-// CTAs (prefix splits) per (query tile, head): as many of 4, 2, 1 as run at once (three CTAs per SM) and
-// leave each CTA pages enough.  One CTA without path keys writes its rows directly, so a short prefix is
-// not split then.  us, 1 / 2 / 4 CTAs, 128-wide heads: 128 pairs of 8 pages with path keys 21.8 / 18.1 / 25.5,
-// 256 of 8 26.6 / 32.7 / 42.0, 64 of 8 21.8 / 14.4 / 14.0, 64 of 5 17.1 / 12.9 / 13.9, 32 of 5 13.8 / 10.8 / 10.3;
-// causal without: 128 of 4 9.2 / 11.7 / 21.2, 256 of 8 17.5 / 22.2 / 36.8; 64-wide heads: 48 of 4 6.6 / 7.4 / 7.3,
-// 72 of 6 8.6 / 8.5 / 8.0, 192 of 16 19.6 / 16.9 / 19.5; 32-wide: 16 of 4 7.1 / 7.5 / 5.6.
-int attention_splits(long long pairs, int pages, bool paths, int sms) {
+// CTAs (prefix splits) per (query tile, head) of the attention operator, 1, 2 or 4, and the pages of a split.
+//
+// Up to 256 tokens, where a row of the GEMMs does not depend on the call's other tokens, a query's result does
+// not either: the splits' boundaries come from the prefix, the number of heads and whether there are path keys.
+// As many as run at once (three CTAs per SM) for 128 queries, of a short prefix for 256.  One CTA without path
+// keys writes its rows directly, so a short prefix is not split then.  us of kernel, 1 / 2 / 4 CTAs, 32 heads of
+// 128 with path keys: 128 queries, 2 pages 13.4 / 10.3 / -, 4 pages - / 11.9 / 13.1, 8 pages 21.8 / 14.4 / 14.6; 10
+// queries, 8 pages - / 14.9 / 11.0; 200 queries, 4 pages - / 14.7 / 21.2, 8 pages - / 18.5 / 25.4 (the boundaries of 128
+// queries cost most there); 4 heads of 32, 4 pages, 120 queries - / 8.5 / 6.2; no path keys: 250 queries, 4 pages
+// 9.3 / 13.3 / 22.4.
+//
+// More tokens: as many as run at once and leave each CTA pages enough, the pages each tile sees balanced over
+// them (pages = 0).  us, 1 / 2 / 4 CTAs, 128-wide heads: 256 pairs of 8 pages with path keys 26.6 / 32.7 / 42.0,
+// causal without 17.5 / 22.2 / 36.8; 64-wide heads: 72 of 6 8.6 / 8.5 / 8.0, 192 of 16 19.6 / 16.9 / 19.5.
+struct AttnSplits {
+  int n, pages;
+};
+AttnSplits attention_splits(int T, int n_heads, int pages, bool paths, int sms) {
   const long long room = 3LL * sms;
-  const int least4 = paths ? (8 * pairs <= 3LL * sms ? 4 : 8) : 4 * pairs <= sms ? 4 : 6;
-  if (4 * pairs <= room && pages >= least4) return 4;
-  return 2 * pairs <= room && pages >= (paths ? 2 : 8) ? 2 : 1;
+  if (T <= 256) {
+    int n = pages > 4 || (pages > 2 && 16LL * n_heads <= room) ? 4 : pages > 1 ? 2 : 1;
+    if (!paths && pages < 8) n = 1;
+    while (n > 1 && 2LL * n * n_heads > room) n /= 2;
+    return {n, std::max(1, (pages + n - 1) / n)};
+  }
+  const long long pairs = (long long)((T + ATT_QTILE - 1) / ATT_QTILE) * n_heads;
+  const int least4 = paths ? (8 * pairs <= room ? 4 : 8) : 4 * pairs <= sms ? 4 : 6;
+  if (4 * pairs <= room && pages >= least4) return {4, 0};
+  return {2 * pairs <= room && pages >= (paths ? 2 : 8) ? 2 : 1, 0};
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -181,7 +199,8 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
   }
   bool paths = false;
   for (int t = 0; h_n_path && t < T; ++t) paths |= h_n_path[t] > 0;
-  const int S = attention_splits((long long)nqt * n_heads, pages, paths, current_grid());
+  const AttnSplits splits = attention_splits(T, n_heads, pages, paths, current_grid());
+  const int S = splits.n;
   const int d = n_heads * head_dim;
   CUtensorMap mk, mv;
   char eb[256];
@@ -198,7 +217,7 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
   a.kv_rows = cache_rows;
   a.n_qtiles = nqt;
   a.max_pages = std::max(1, pages);
-  a.chunks_per_split = 0;
+  a.chunks_per_split = splits.pages;
   a.max_splits = S;
   a.out = static_cast<__nv_bfloat16*>(d_out);
   a.direct = S == 1 && !paths;

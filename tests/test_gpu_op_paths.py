@@ -132,6 +132,34 @@ def test_attention_paths(ats, H, hd, P, T, paths):
     assert bool(((out - ref).abs() <= 2.0 ** -8 * ref.abs() + 2.0 ** -11 * mag + 1e-5).all())
 
 
+# up to 256 tokens a query's result is that of its own keys, whatever else is in the call: fewer queries, other
+# tiles, neighbours that see more or less of the prefix; the numbers of heads and pages that give one, two and
+# four splits
+@pytest.mark.parametrize("H,hd,P", [(32, 128, 448), (32, 128, 512), (32, 64, 200), (4, 32, 250), (12, 64, 1000), (60, 32, 600),
+                                    (120, 32, 300), (2, 64, 2500)])
+def test_attention_result_does_not_depend_on_the_other_queries(ats, H, hd, P):
+    rng = np.random.default_rng(P)
+    T, d, n = 256, H * hd, (P + 63) // 64
+    pages = rng.permutation(n + 3)[:n]
+    rows = 64 * (n + 3) + 40
+    q, kc = _randn((T, d), 1), _randn((rows, d), 2)
+    vc = _randn((rows, d), 3).to(torch.float16)
+    vis = np.where(rng.random(T) < 0.5, P, rng.integers(0, P + 1, size=T)).astype(np.int32)
+    n_path = rng.integers(0, 5, size=T).astype(np.int32)
+    path = rng.integers(0, rows, size=(T, 4)).astype(np.int32)
+    n_path[[7, 60]] = 4   # (path keys in every call of the first kind)
+
+    def run(i, paths):
+        i = np.asarray(i)
+        return ats.op_attention(q[torch.from_numpy(i).cuda()].contiguous(), kc, vc, H, hd, P, pages, vis[i],
+                                path[i] if paths else None, n_path[i] if paths else None)
+
+    for paths in (True, False):
+        full = run(np.arange(T), paths)
+        for i in ([7], np.arange(10), np.concatenate([[7], rng.permutation(T)[:63]]), np.arange(120), np.arange(50, 250)):
+            assert torch.equal(run(i, paths), full[torch.as_tensor(i).cuda()])
+
+
 # whole-vocabulary log-sum-exp (FULL normalisation): one token tile of every width, several; a partial last
 # weight tile; enough tiles for the CTA pairs (an odd and an even count)
 @pytest.mark.parametrize("V,users,N,gamma", [(1200, 1, 7, 1), (1200, 3, 17, 1), (2000, 2, 40, 1), (1200, 1, 80, 3),
