@@ -299,7 +299,8 @@ atspeed_status atspeed_op_rmsnorm(atspeed_stream stream, const float *d_h, const
  * causal prefill).  out bf16 [T][H*hd].  Among calls of up to 256 tokens that have path keys, and among
  * those that have none, a token's result depends on its own keys and P alone, not on the call's other
  * tokens (as up to 256 tokens a row of the GEMMs does not); larger calls group the softmax's sums by their
- * size.  d_part: fp32 scratch of atspeed_op_attention_scratch(T,H,hd,P). */
+ * size.  d_part: scratch of atspeed_op_attention_scratch(T,H,hd,P) bytes, 4-byte
+ * aligned (the call's tables, where they are more than kernel parameters hold: about 24 bytes a token). */
 size_t atspeed_op_attention_scratch(int T, int n_heads, int head_dim, int P);
 atspeed_status atspeed_op_attention(atspeed_stream stream, const void *d_q, const void *d_kcache, const void *d_vcache,
                                     int cache_rows, int T, int n_heads, int head_dim, int P, const int32_t *h_pages,

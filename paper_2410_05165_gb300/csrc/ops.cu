@@ -169,12 +169,13 @@ atspeed_status atspeed_op_rmsnorm(atspeed_stream stream, const float* d_h, const
 }
 
 size_t atspeed_op_attention_scratch(int T, int n_heads, int head_dim, int P) {
-  const int pages = (P + ATT_PAGE - 1) / ATT_PAGE;
-  const int S = std::max(1, (pages + 1) / 2);
-  const int nqt = (T + ATT_QTILE - 1) / ATT_QTILE;
-  const size_t floats = (size_t)S * T * n_heads * head_dim + (size_t)S * T * n_heads * 2;
-  const size_t ints = (size_t)4 * nqt + (size_t)T * 7 + pages + 1;
-  return floats * 4 + ints * 4 + 256;
+  (void)n_heads;
+  (void)head_dim;
+  AttnArgs a = {};   // the call's tables (used where they are more than kernel parameters hold)
+  a.T = T;
+  a.n_qtiles = (T + ATT_QTILE - 1) / ATT_QTILE;
+  a.max_pages = std::max(1, (P + ATT_PAGE - 1) / ATT_PAGE);
+  return attn_tables(a, nullptr, true) * sizeof(int);
 }
 
 atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, const void* d_kcache, const void* d_vcache,

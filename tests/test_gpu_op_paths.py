@@ -1,5 +1,7 @@
 """Each path of the operators' dispatch at the sizes where it can go wrong (edges of tiles, groups and
 cluster sizes, the smallest and largest of a range, general alignments) against fp64."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -151,6 +153,25 @@ def test_attention_paths(ats, H, hd, P, T, paths):
         mag = mag + torch.einsum("htj,tjhd->thd", w[:, :, P:], pv.abs())
     # the weights are rounded to fp16 (2^-11), the result to bf16
     assert bool(((out - ref).abs() <= 2.0 ** -8 * ref.abs() + 2.0 ** -11 * mag + 1e-5).all())
+
+
+# tables on both sides of what kernel parameters hold: nothing beyond the scratch that the call asks for is written
+@pytest.mark.parametrize("T", [1200, 1300])
+def test_attention_scratch(ats, T):
+    H, hd, P = 2, 32, 70
+    d, rows, rng = H * hd, 64 * 4, np.random.default_rng(T)
+    q, kc = _randn((T, d), 1), _randn((rows, d), 2)
+    vc = _randn((rows, d), 3).to(torch.float16)
+    pages, vis = np.array([2, 0], np.int32), rng.integers(0, P + 1, size=T).astype(np.int32)
+    n_path, path = rng.integers(0, 5, size=T).astype(np.int32), rng.integers(0, rows, size=(T, 4)).astype(np.int32)
+    lib = ats.load()
+    size = lib.atspeed_op_attention_scratch(T, H, hd, P)
+    part, out = torch.full((size + 256,), 7, dtype=torch.uint8, device="cuda"), torch.empty_like(q)
+    ptr = [x.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)) for x in (pages, vis, path, n_path)]
+    assert lib.atspeed_op_attention(torch.cuda.current_stream().cuda_stream, q.data_ptr(), kc.data_ptr(), vc.data_ptr(),
+                                    rows, T, H, hd, P, *ptr, out.data_ptr(), part.data_ptr()) == ats.OK
+    assert bool((part[size:] == 7).all())
+    assert torch.equal(out, ats.op_attention(q, kc, vc, H, hd, P, pages, vis, path, n_path))
 
 
 # up to 256 tokens a query's result is that of its own keys, whatever else is in the call: fewer queries, other

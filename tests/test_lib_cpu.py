@@ -46,3 +46,11 @@ def test_create_rejects_null_arguments(lib):
     assert st == -1
     lib.atspeed_last_error.restype = ctypes.c_char_p
     assert b"null" in lib.atspeed_last_error(None)
+
+
+def test_attention_scratch_holds_the_tables_alone(lib):
+    """Page, visibility and path-key tables of a call; its partial sums never pass through memory."""
+    lib.atspeed_op_attention_scratch.restype = ctypes.c_size_t
+    for T, H, hd, P in ((1, 1, 32, 0), (120, 32, 128, 512), (1000, 32, 128, 1000)):
+        tables = 4 * (6 * T + P // 64 + T // 16 + 8)
+        assert 24 * T <= lib.atspeed_op_attention_scratch(T, H, hd, P) <= tables
