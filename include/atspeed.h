@@ -270,12 +270,13 @@ atspeed_status atspeed_op_gemm(atspeed_stream stream, const void *d_W, const voi
 atspeed_status atspeed_op_gemm_noalloc(atspeed_stream stream, const void *d_W, const void *d_X, int M, int K, int T,
                                        int x_rows, float *d_Y, int ldy, int accumulate);
 
-/* Device-side failures of the op GEMMs above (atspeed_op_gemm, atspeed_op_gemm_swiglu,
- * atspeed_op_gemm_noalloc).  Their launches return ATSPEED_OK once enqueued; a bounded wait inside
- * the kernel that gives up (a copy or a peer CTA that never arrives) does not trap but sets an error
- * word in the call's scratch, which stays set (sticky) across later calls until this function reads
- * it.  Synchronises `stream`, reads and clears the word of the workspace d_ws (or, with d_ws = NULL,
- * of the allocation-free entry point's scratch on the current device) and returns ATSPEED_OK,
+/* Device-side failures of the op GEMMs (atspeed_op_gemm, atspeed_op_gemm_swiglu,
+ * atspeed_op_gemm_noalloc) and of atspeed_op_attention.  Their launches return ATSPEED_OK once
+ * enqueued; a bounded wait inside the kernel that gives up (a copy or a peer CTA that never arrives)
+ * does not trap but sets an error word in the call's workspace (for the allocation-free entry point
+ * and the attention: a word of this library on the device), which stays set (sticky) across later calls
+ * until this function reads it.  Synchronises `stream`, reads and clears the word of the workspace d_ws
+ * (or, with d_ws = NULL, the library's words on the current device) and returns ATSPEED_OK,
  * ATSPEED_E_TIMEOUT (a bounded wait gave up: the outputs of the calls since the last check are not
  * valid) or ATSPEED_E_CUDA (the synchronisation or the read failed).  Not part of the paper: it is
  * how the stateless operators report device errors. */

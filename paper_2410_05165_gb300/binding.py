@@ -360,7 +360,8 @@ def op_gemm_noalloc(W: torch.Tensor, X: torch.Tensor, T: int, Y: Optional[torch.
 
 def op_status(noalloc: bool = False, stream=None) -> int:
     """atspeed_op_status: synchronises, reads and clears the device error word of the op GEMMs'
-    workspace (or of the allocation-free scratch); returns the status code (0 = no device error)."""
+    workspace (noalloc: those of the allocation-free scratch and of the attention); returns the status
+    code (0 = no device error)."""
     ws = None if noalloc else op_workspace().data_ptr()
     return int(load().atspeed_op_status(_stream(stream), ws))
 

@@ -98,6 +98,9 @@ struct AttClusterSink {
   }
 };
 
+// Set by a bounded wait of the operator's kernel that gave up; sticky until atspeed_op_status reads it.
+__device__ unsigned int g_attn_err;
+
 // The call's tables in the kernel's parameters (NTAB ints), or in memory (NTAB = 0).
 template <int NTAB>
 struct AttTables {
@@ -109,6 +112,7 @@ __global__ void __launch_bounds__(128, 3)
     attn_cluster_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv,
                         const AttnArgs args, const int S, const int paths, const __grid_constant__ AttTables<NTAB> tab) {
   AttnArgs a = args;
+  a.err = &g_attn_err;
   if constexpr (NTAB > 0) attn_tables(a, tab.v, paths);
   using CC = AttClusterCfg<HD>;
   extern __shared__ uint8_t smem_raw[];
@@ -346,6 +350,11 @@ cudaError_t attn_cluster_launch(AttnArgs a, const CUtensorMap& mk, const CUtenso
     case 128: return launch_cluster_hd<128>(a, mk, mv, S, tables, n, paths, d_tables, st);
   }
   return cudaErrorInvalidValue;
+}
+
+unsigned int* attn_err_word() {
+  void* p = nullptr;
+  return cudaGetSymbolAddress(&p, g_attn_err) == cudaSuccess ? static_cast<unsigned int*>(p) : nullptr;
 }
 
 }  // namespace atspeed

@@ -76,4 +76,7 @@ __host__ __device__ inline size_t attn_tables(AttnArgs& a, const int* base, bool
 cudaError_t attn_cluster_launch(AttnArgs a, const CUtensorMap& mk, const CUtensorMap& mv, int S, const int* tables,
                                 size_t n, bool paths, int* d_tables, cudaStream_t st);
 
+// The operator's error word on the current device (ATSPEED_DEV_ERR_* bits); null if it cannot be found.
+unsigned int* attn_err_word();
+
 }  // namespace atspeed

@@ -222,7 +222,6 @@ atspeed_status atspeed_op_attention(atspeed_stream stream, const void* d_q, cons
   a.max_splits = S;
   a.out = static_cast<__nv_bfloat16*>(d_out);
   a.direct = S == 1 && !paths;
-  a.err = nullptr;
   std::vector<int> host(attn_tables(a, nullptr, paths), 0);
   AttnArgs at = a;
   attn_tables(at, host.data(), paths);
@@ -279,23 +278,29 @@ atspeed_status atspeed_op_gemm_noalloc(atspeed_stream stream, const void* d_W, c
   return gemm_status(gemm_launch(a, s, kNoAllocGrid, (cudaStream_t)stream, false, eb, sizeof eb));
 }
 
-/* See include/atspeed.h.  Reads (and clears) the error word that the op GEMMs' bounded waits set. */
+/* See include/atspeed.h.  Reads (and clears) the error words that the operators' bounded waits set. */
 atspeed_status atspeed_op_status(atspeed_stream stream, void* d_ws) {
-  unsigned int* word = nullptr;
+  unsigned int* words[2] = {nullptr, nullptr};
   if (d_ws) {
-    word = scratch_from(d_ws, current_grid()).err;
+    words[0] = scratch_from(d_ws, current_grid()).err;
   } else {
     void* base = noalloc_base();
-    if (!base) return ATSPEED_E_CUDA;
-    word = noalloc_err_word(base);
+    words[1] = attn_err_word();
+    if (!base || !words[1]) return ATSPEED_E_CUDA;
+    words[0] = noalloc_err_word(base);
   }
   cudaStream_t st = (cudaStream_t)stream;
   if (cudaStreamSynchronize(st) != cudaSuccess) return ATSPEED_E_CUDA;
-  unsigned int v = 0;
-  if (cudaMemcpy(&v, word, sizeof v, cudaMemcpyDeviceToHost) != cudaSuccess) return ATSPEED_E_CUDA;
-  if (v == 0) return ATSPEED_OK;
-  if (cudaMemset(word, 0, sizeof v) != cudaSuccess) return ATSPEED_E_CUDA;
-  return (v & ATSPEED_DEV_ERR_TIMEOUT) ? ATSPEED_E_TIMEOUT : ATSPEED_E_CUDA;
+  unsigned int all = 0;
+  for (unsigned int* word : words) {
+    unsigned int v = 0;
+    if (!word) continue;
+    if (cudaMemcpy(&v, word, sizeof v, cudaMemcpyDeviceToHost) != cudaSuccess) return ATSPEED_E_CUDA;
+    if (v != 0 && cudaMemset(word, 0, sizeof v) != cudaSuccess) return ATSPEED_E_CUDA;
+    all |= v;
+  }
+  if (all == 0) return ATSPEED_OK;
+  return (all & ATSPEED_DEV_ERR_TIMEOUT) ? ATSPEED_E_TIMEOUT : ATSPEED_E_CUDA;
 }
 
 }  // extern "C"

@@ -172,6 +172,7 @@ def test_attention_scratch(ats, T):
                                     rows, T, H, hd, P, *ptr, out.data_ptr(), part.data_ptr()) == ats.OK
     assert bool((part[size:] == 7).all())
     assert torch.equal(out, ats.op_attention(q, kc, vc, H, hd, P, pages, vis, path, n_path))
+    assert ats.op_status(noalloc=True) == ats.OK   # (no bounded wait gave up: the attention's word is among these)
 
 
 # up to 256 tokens a query's result is that of its own keys, whatever else is in the call: fewer queries, other
