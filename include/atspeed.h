@@ -293,12 +293,11 @@ atspeed_status atspeed_op_rmsnorm(atspeed_stream stream, const float *d_h, const
 
 /* Tree attention of T query tokens of ONE user over a paged prefix of length P plus per-token path
  * keys (Sec. 3.3, App. A.3.1).  q bf16 [T][H*hd]; K cache bf16 [rows][H*hd]; V cache fp16
- * [rows][H*hd] holding bf16-rounded values (the library's own layout: P V runs in fp16 with P split
- * into two fp16 halves); prefix row p of the
- * user is cache row 64*h_pages[p/64] + p%64; token t also attends to the n_path[t] <= 4 cache rows
- * path_rows[t][0..], and sees prefix positions < vis[t] (vis[t] = P for tree nodes, t+1 for a
- * causal prefill).  out bf16 [T][H*hd].  Among calls of up to 256 tokens that have path keys, and among
- * those that have none, a token's result depends on its own keys and P alone, not on the call's other
+ * [rows][H*hd] holding bf16-rounded values (the library's own layout: P V runs in fp16, with P rounded to
+ * fp16); prefix row p of the user is cache row 64*h_pages[p/64] + p%64; token t also attends to the
+ * n_path[t] <= 4 cache rows path_rows[t][0..], and sees prefix positions < vis[t] (vis[t] = P for tree nodes,
+ * t+1 for a causal prefill).  out bf16 [T][H*hd].  Among calls of up to 256 tokens that have path keys, and
+ * among those that have none, a token's result depends on its own keys and P alone, not on the call's other
  * tokens (as up to 256 tokens a row of the GEMMs does not); larger calls group the softmax's sums by their
  * size.  d_part: scratch of atspeed_op_attention_scratch(T,H,hd,P) bytes, 4-byte
  * aligned (the call's tables, where they are more than kernel parameters hold: about 24 bytes a token). */

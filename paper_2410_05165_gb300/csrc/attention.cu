@@ -1,8 +1,8 @@
-// Shared-prefix tree attention: TMA-staged K/V pages, tensor cores (mma.sync m16n8k16: bf16 Q K^T;
-// P V with P split into two fp16 halves and V in fp16) with an fp32 online softmax, prefix split across
-// CTAs.  The one-kernel-per-op schedule's prefix kernel leaves the splits to a combine kernel, which merges
-// them with each node's path keys (ancestors + self, at most 4); the operator's kernel does both, with the
-// splits of a tile in one cluster.
+// Shared-prefix tree attention: TMA-staged K/V pages, tensor cores (mma.sync m16n8k16: bf16 Q K^T; P V in
+// fp16, with P rounded to fp16 once, 2^-11 of a weight, and V exact) with an fp32 online softmax, prefix split
+// across CTAs.  The one-kernel-per-op schedule's prefix kernel leaves the splits to a combine kernel, which
+// merges them with each node's path keys (ancestors + self, at most 4); the operator's kernel does both, with
+// the splits of a tile in one cluster.
 #include <cudaTypedefs.h>
 #include <math.h>
 #include <stdio.h>
@@ -49,12 +49,13 @@ __global__ void __launch_bounds__(128) attn_combine_kernel(const AttnArgs a) {
 }
 
 // ---- the operator's attention: one kernel, the prefix splits of a (query tile, head) in one cluster
-// S CTAs (1, 2 or 4) share the tile's visible pages; their partials (o, m, l) meet in distributed shared
-// memory -- 16-query group g belongs to CTA g mod S, every CTA stores its rows of the group there -- and
-// the owner merges them with the queries' path keys.  Against the two kernels above (partials through
-// global memory, fixed splits of two pages, most of them empty for the early tiles of a causal prefill):
-// causal 1000 tokens x 32 heads of 128 61 + 30 us before, 38 now, the call 106 -> 39 us; a tree of 120 tokens
-// over 512 keys 65 -> 34 us a call (host-bound: the kernel takes 14).
+// S CTAs (1, 2 or 4) share the prefix's pages (ranges that do not depend on the tile, or the tile's visible pages
+// evenly: chunks_per_split); their partials (o, m, l) meet in distributed shared memory -- 16-query group g
+// belongs to CTA g mod S, every CTA stores its rows of the group there -- and the owner merges them with the
+// queries' path keys.  Against the two kernels above (partials through global memory, splits of two pages, most
+// of them empty for the early tiles of a causal prefill): causal 1000 tokens x 32 heads of 128 61 + 30 us
+// before, 38 now, the call 106 -> 40 us; a tree of 120 tokens over 512 keys 65 -> 36 us a call (host-bound: the
+// kernel takes 14.6).
 // Bound: latency for few queries (Q, K/V and path-key round trips); for many, a step's shared-memory
 // reads (every warp reads the whole K/V tile through ldmatrix) and its MMAs, which take about as long.
 template <int HD>

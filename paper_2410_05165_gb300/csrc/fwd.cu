@@ -394,10 +394,6 @@ __device__ __forceinline__ bool attn_phase(const FwdParams& p, int l, uint8_t* a
     if (a.direct) continue;
     const int S_u = a.user_splits[a.qt_user[tile]];
     if (split >= S_u) continue;
-    // every split publishes its partials and waits for the others of (tile, h) -- all items run in
-    // one round (2 G work slots), or the awaited ones in a later round, never an earlier one -- then
-    // split s merges query groups s, s + S_u, ...  The counter only grows during a launch: layer l
-    // completes at S_u * (l + 1).
     // publish this split's partials (every thread's are stored before the barrier, thread 0's release
     // carries them); then split s merges query groups s, s + S_u, ... once all splits of (tile, h) are
     // there -- all items run in one round (2 G work slots), or the awaited ones in a later round, never
