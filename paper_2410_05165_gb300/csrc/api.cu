@@ -62,7 +62,8 @@ struct Fail {
 struct ModelRt {
   bool present = false;
   bool per_op = false;   // this model's forward runs one kernel per op (else one persistent launch)
-  int grid = 0;          // CTAs of the current forward's GEMM work splits (both schedules, so both give the same bits)
+  int grid = 0;          // CTAs of the current forward
+  int split = 0;         // CTAs that its split GEMM tiles are split for (both schedules, so both give the same bits)
   int cps = 2;           // prefix pages per attention split of its tree forwards (fixed per context)
   int layers = 0, d = 0, H = 0, hd = 0, ffn = 0, V = 0;
   float eps = 1e-6f, theta = 1e4f;
@@ -110,12 +111,12 @@ struct ModelRt {
 // CTAs of a forward of T tokens.  One token tile (256 tokens): min(SMs, gate/up weight tiles), so that a
 // small model takes one whole gate/up tile per CTA with no split sums, and every grid barrier spans fewer
 // CTAs (4 layers, 48 tiles, 128 tokens, us on 48 / 96 / 152 CTAs: 184 / 213 / 262).  More token tiles give
-// work to more CTAs: short gate/up tiles (<= 16 k-blocks) still whole, as evenly as that goes (the sum of a
-// split tile costs as much as the tile), long ones on every SM.  us on the weight tiles' count of CTAs ->
-// here: the 4-layer model, 512 tokens 297 -> 250 (152 CTAs: 345), 1000 536 -> 342 (403), 3000 1254 -> 566
-// (686), 4000 1544 -> 769 (814); 2 layers of 2048 (88 tiles of 32 k-blocks), 512 tokens 252 -> 234, 1000 455
-// -> 351 (118 whole-tile CTAs: 405), 4000 1400 -> 910; the 2-layer d 128 model (8 tiles), 1000 tokens 306 ->
-// 142, 4000 1012 -> 161 (the attention's items ask for at least 64 there: 32 CTAs 151 at 1000 tokens).
+// their whole weight tiles to more CTAs (split tiles stay split for as many as one token tile has, so the
+// bits do not depend on this): short gate/up tiles (<= 16 k-blocks) as evenly as that goes, long ones over
+// every SM.  us of a prefill call on the weight tiles' count of CTAs -> here: the 4-layer model, 512 tokens
+// 345 -> 315, 1000 605 -> 449, 4000 1707 -> 810; 4 layers of 2048 (88 tiles of 32 k-blocks), 512 tokens 529 ->
+// 510, 1000 941 -> 806 (on 118 CTAs 878), 3000 2100 -> 1535; the 2-layer d 128 model (8 tiles), 1000 tokens 446
+// -> 208, 4000 1444 -> 240 (the attention's items ask for at least 64 CTAs there).
 int forward_ctas(const ModelRt& m, int T, int sms) {
   const int weight_tiles = 2 * m.ffn / 128, tiles = weight_tiles * std::max(1, (T + 255) / 256);
   int G = tiles;
@@ -629,7 +630,7 @@ struct ProfScope {
   }
 };
 
-void gemm(atspeed_ctx* c, const GemmArgs& a, cudaStream_t st, int kind, int grid) {
+void gemm(atspeed_ctx* c, const GemmArgs& a, cudaStream_t st, int kind, int split, int grid) {
   char eb[256] = {0};
   // algorithmic bytes: weights once, activations in, outputs out
   const double out_b = a.epi == EPI_F32 ? 4.0 * a.M : a.epi == EPI_RESID ? 8.0 * a.M
@@ -639,7 +640,7 @@ void gemm(atspeed_ctx* c, const GemmArgs& a, cudaStream_t st, int kind, int grid
   // the whole-vocabulary head takes the operators' kernels and the whole GPU, the forward's GEMMs the
   // work split they share with the persistent kernel (33024 rows of 4096: 4 tokens 50 -> 45 us, 6.0 TB/s;
   // 960 tokens 187 -> 162 us, 1.6 PFLOP/s)
-  cudaError_t e = a.epi != EPI_LSE ? gemm_launch(a, c->gs, grid, st, c->pdl && !c->prof, eb, sizeof eb)
+  cudaError_t e = a.epi != EPI_LSE ? gemm_launch(a, c->gs, split, grid, st, c->pdl && !c->prof, eb, sizeof eb)
                   : gemm_cluster_fits(a, c->gemm_grid)
                       ? gemm_cluster_launch(a, c->err_word, c->gemm_grid, st, eb, sizeof eb)
                       : gemm_pair_launch(a, c->gs, c->gemm_grid, st, eb, sizeof eb);
@@ -659,6 +660,7 @@ void forward(atspeed_ctx* c, ModelRt& m, const FwdPlan& p, cudaStream_t st) {
     throw Fail{ATSPEED_E_SHAPE};
   }
   m.grid = forward_ctas(m, T, c->fwd_grid);
+  m.split = forward_ctas(m, 1, c->fwd_grid);
   const int nqt = (int)p.qt_t0.size();
   if (nqt > m.max_qt || (int)p.splits.size() > c->lim.max_users || (int)p.out_rows.size() > m.Tcap) {
     set_err(c, "forward plan exceeds capacity (%d query tiles, %zu users, %zu rows)", nqt, p.splits.size(),
@@ -702,6 +704,7 @@ void forward(atspeed_ctx* c, ModelRt& m, const FwdPlan& p, cudaStream_t st) {
     f.L = m.layers;
     f.eps = m.eps;
     f.G = m.grid;
+    f.Gs = m.split;
     f.maps = m.maps;
     f.attn_norm = m.d_attn_norm;
     f.mlp_norm = m.d_mlp_norm;
@@ -795,7 +798,7 @@ void forward(atspeed_ctx* c, ModelRt& m, const FwdPlan& p, cudaStream_t st) {
     g.q_out = m.q;
     g.k_cache = m.kc + per * l;
     g.v_cache = m.vc + per * l;
-    gemm(c, g, st, 0, m.grid);
+    gemm(c, g, st, 0, m.split, m.grid);
     AttnArgs a = {};
     a.T = T;
     a.n_heads = m.H;
@@ -843,7 +846,7 @@ void forward(atspeed_ctx* c, ModelRt& m, const FwdPlan& p, cudaStream_t st) {
     g.X_rows = m.Xrows;
     g.out_f32 = m.h;
     g.ldo = m.d;
-    gemm(c, g, st, 1, m.grid);
+    gemm(c, g, st, 1, m.split, m.grid);
     g = GemmArgs{};
     folded(g);
     g.ssq_in = m.ssq;
@@ -856,7 +859,7 @@ void forward(atspeed_ctx* c, ModelRt& m, const FwdPlan& p, cudaStream_t st) {
     g.X_rows = m.Xrows;
     g.out_bf16 = m.act;
     g.ldo = m.ffn;
-    gemm(c, g, st, 2, m.grid);
+    gemm(c, g, st, 2, m.split, m.grid);
     g = GemmArgs{};
     folded(g);
     g.epi = EPI_RESNORM;
@@ -873,7 +876,7 @@ void forward(atspeed_ctx* c, ModelRt& m, const FwdPlan& p, cudaStream_t st) {
     g.X_rows = m.Xrows;
     g.out_f32 = m.h;
     g.ldo = m.d;
-    gemm(c, g, st, 3, m.grid);
+    gemm(c, g, st, 3, m.split, m.grid);
   }
   const int n_out = (int)p.out_rows.size();
   CK(rmsnorm_rows_launch(m.h, m.rows_sel, n_out, m.final_norm, m.d, m.eps, m.x, m.d, st, pdl));
@@ -888,7 +891,7 @@ void forward(atspeed_ctx* c, ModelRt& m, const FwdPlan& p, cudaStream_t st) {
   g.X_rows = m.Xrows;
   g.out_f32 = m.logits + (size_t)p.logit_row_base * ITEM_ROWS;
   g.ldo = ITEM_ROWS;
-  gemm(c, g, st, 4, m.grid);
+  gemm(c, g, st, 4, m.split, m.grid);
 }
 
 // FULL normalisation (whole-vocabulary log-softmax, then the trie mask): log-sum-exp over the whole
@@ -910,7 +913,7 @@ void full_lse(atspeed_ctx* c, ModelRt& m, const bf16* X, int X_rows, int n, floa
   g.X_rows = X_rows;
   g.lse_part = m.lse_part;
   g.lse_ld = m.lse_ld;
-  gemm(c, g, st, 4, m.grid);
+  gemm(c, g, st, 4, m.split, m.grid);
   CK(lse_combine_launch(m.lse_part, m.lse_ld, (m.V + 127) / 128, n, lse_out, st));
   c->n_launch += 1;
 }

@@ -27,6 +27,7 @@ struct FwdParams {
   int d, H, hd, ffn, L;
   float eps;
   int G;          // CTAs (one per SM, all co-resident)
+  int Gs;         // CTAs that split GEMM tiles are split for (<= G)
   const CUtensorMap* maps;
   // norms, embedding (bf16)
   const __nv_bfloat16* const* attn_norm;  // [L] device pointers

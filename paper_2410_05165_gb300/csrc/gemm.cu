@@ -50,7 +50,6 @@ struct KParams {
   GemmArgs a;
   int m_tiles, n_tiles, kb;
   WorkSplit w;   // whole tiles per CTA + stream-K over the remaining tiles
-  int G;
   int up_row0;
   float* ws;
   int* counters;
@@ -357,7 +356,7 @@ cudaError_t launch_t(const CUtensorMap& ma, const CUtensorMap& mb, const KParams
   const cudaError_t e = smem_attr_once(attr_done, gemm_kernel<BN, EPI>, C::SMEM);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kp.G);
+  cfg.gridDim = dim3(kp.w.Gw);
   cfg.blockDim = dim3(192);
   cfg.dynamicSmemBytes = C::SMEM;
   cfg.stream = st;
@@ -469,7 +468,7 @@ cudaError_t gemm_check(const GemmArgs& a, int max_tiles, char* eb, size_t el) {
   return cudaSuccess;
 }
 
-cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaStream_t stream, bool pdl,
+cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int split, int grid, cudaStream_t stream, bool pdl,
                         char* eb, size_t el) {
   const cudaError_t ce = gemm_check(a, s.max_tiles, eb, el);
   if (ce != cudaSuccess) return ce;
@@ -481,9 +480,9 @@ cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaS
   kp.up_row0 = a.epi == EPI_SWIGLU ? a.M / 2 : 0;
   kp.kb = a.K / BK;
   const long long tiles = (long long)kp.m_tiles * kp.n_tiles;
-  kp.G = gemm_work_ctas(tiles, kp.kb, grid);
-  kp.w = work_split((int)tiles, kp.kb, kp.G);
-  if (s.ws_bytes < gemm_ws_bytes(kp.G)) {
+  const int G = gemm_work_ctas(tiles, kp.kb, split);
+  kp.w = work_split((int)tiles, kp.kb, G, grid);
+  if (s.ws_bytes < gemm_ws_bytes(G)) {
     snprintf(eb, el, "gemm: workspace too small");
     return cudaErrorInvalidValue;
   }

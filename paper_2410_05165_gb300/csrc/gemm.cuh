@@ -87,7 +87,8 @@ constexpr cudaError_t kGemmMapError = cudaErrorInvalidDevicePointer;
 cudaError_t gemm_check(const GemmArgs& a, int max_tiles, char* errbuf, size_t errlen);
 
 // Encodes the tensor maps and launches.  `pdl` enables programmatic dependent launch.
-cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int grid, cudaStream_t stream, bool pdl,
+// Split tiles are split for `split` CTAs (the bits depend on it), whole tiles go to `grid` >= split CTAs.
+cudaError_t gemm_launch(const GemmArgs& a, const GemmScratch& s, int split, int grid, cudaStream_t stream, bool pdl,
                         char* errbuf, size_t errlen);
 
 // The operators' GEMM with few output tiles (gemm_cluster.cu): EPI_F32, EPI_RESID, EPI_SWIGLU and EPI_LSE,

@@ -10,23 +10,25 @@ constexpr int GEMM_BM = 128;   // weight rows per tile (MMA M)
 constexpr int GEMM_WS_SLOT_FLOATS = 256 * 128;
 
 // ---- work split of a tiled GEMM over G CTAs (tiles of kb k-blocks)
-// Each CTA takes q = tiles / G whole tiles; the first r = tiles % G tiles are split by k-blocks into
+// q = tiles / G whole tiles per CTA; the first r = tiles % G tiles are split by k-blocks into
 // G equal contiguous unit ranges (stream-K; unit = one tile's k-block).  A CTA works on its
-// stream-K units first and then on its whole tiles r + c, r + c + G, ..., r + c + (q - 1) G, so the
+// stream-K units first and then on its whole tiles (every G-th from r + c on), so the
 // partial sums of the split tiles are published early and the tail after the last MMA is
 // whole-tile epilogues.  Whole tiles go round robin: at each step the grid works on G consecutive
 // tiles, i.e. (the token-tile index varying fastest) on every token tile of a few weight row tiles,
 // so each weight tile is read from DRAM about once per step and shared through L2 by the CTAs
 // that need it, where a contiguous range per CTA would have one CTA read it once per token tile.
-// With tiles < G (q = 0) this is plain stream-K over all tiles.
+// With tiles < G (q = 0) this is plain stream-K over all tiles.  A grid of more than G CTAs takes the whole
+// tiles all over (those without stream-K units first); the sums stay those of G.
 struct WorkSplit {
   int tiles, kb, q, r;
   int Usk;         // stream-K units: r * kb (G * Usk fits 32 bits: r < G <= SMs, kb <= 256)
   int Gsk;         // CTAs that get stream-K units: min(G, Usk)
-  int G;           // CTAs that take work (any others of the grid idle in this GEMM)
+  int Gw, off;     // the q G whole tiles go round robin over Gw CTAs (those that take work) from CTA `off` on
 };
 
-__host__ __device__ inline WorkSplit work_split(int tiles, int kb, int G) {
+// G: the CTAs that the remainder is split for; grid >= G: the CTAs that take whole tiles.
+__host__ __device__ inline WorkSplit work_split(int tiles, int kb, int G, int grid) {
   WorkSplit w;
   w.tiles = tiles;
   w.kb = kb;
@@ -34,7 +36,8 @@ __host__ __device__ inline WorkSplit work_split(int tiles, int kb, int G) {
   w.r = tiles - w.q * G;
   w.Usk = w.r * kb;
   w.Gsk = w.Usk < G ? w.Usk : G;
-  w.G = G;
+  w.off = grid > G ? w.Gsk : 0;   // CTAs without stream-K units first
+  w.Gw = grid > G && w.Gsk + w.q * G < grid ? w.Gsk + w.q * G : grid > G ? grid : G;
   return w;
 }
 
@@ -86,25 +89,30 @@ __device__ __forceinline__ void sk_share(const WorkSplit& w, int tile, int c_fir
   lo = (2 * nch * c0 + W) / (2 * W);   // rounded
   hi = (2 * nch * c1 + W) / (2 * W);
 }
+// CTA c's first whole tile
+__device__ __forceinline__ int whole_first(const WorkSplit& w, int c) {
+  return w.r + (c >= w.off ? c - w.off : c - w.off + w.Gw);
+}
 // number of units of CTA c
 __device__ __forceinline__ int cta_units(const WorkSplit& w, int c) {
-  if (c >= w.G) return 0;
+  if (c >= w.Gw) return 0;
   int a, b;
   sk_range(w, c, a, b);
-  return (b - a) + w.q * w.kb;
+  const int t = whole_first(w, c);
+  return (b - a) + (t < w.tiles ? (w.tiles - t + w.Gw - 1) / w.Gw * w.kb : 0);
 }
 // the segments (one tile's contiguous k-blocks [k0, k1)) of CTA c in order
 struct SegIter {
   int u, u1, dp, dp1;
   __device__ __forceinline__ void init(const WorkSplit& w, int c) {
-    if (c >= w.G) {
+    if (c >= w.Gw) {
       u = u1 = 0;
       dp = dp1 = 0;
       return;
     }
     sk_range(w, c, u, u1);
-    dp = w.r + c;                // whole tiles r + c, r + c + G, ... (round robin)
-    dp1 = w.r + w.q * w.G + c;
+    dp = whole_first(w, c);      // and every Gw-th from there on
+    dp1 = w.tiles;
   }
   __device__ __forceinline__ bool next(const WorkSplit& w, int& tile, int& k0, int& k1) {
     if (u < u1) {
@@ -117,7 +125,7 @@ struct SegIter {
     }
     if (dp < dp1) {
       tile = dp;
-      dp += w.G;
+      dp += w.Gw;
       k0 = 0;
       k1 = w.kb;
       return true;

@@ -276,7 +276,7 @@ cudaError_t launch_t(const CUtensorMap& ma, const CUtensorMap& mb, const PairPar
   const cudaError_t e = smem_attr_once(attr_done, gemm_pair_kernel<EPI>, SMEM);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(2 * kp.w.G));
+  cfg.gridDim = dim3((unsigned)(2 * kp.w.Gw));
   cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = SMEM;
   cfg.stream = st;
@@ -301,7 +301,7 @@ cudaError_t gemm_pair_launch(const GemmArgs& a, const GemmScratch& s, int grid, 
   kp.n_tiles = (a.T + BN - 1) / BN;
   kp.m_tiles = (a.M + GEMM_BM - 1) / GEMM_BM;
   kp.kb = a.K / GEMM_BK;
-  kp.w = work_split((kp.m_tiles + 1) / 2 * kp.n_tiles, kp.kb, grid / 2);
+  kp.w = work_split((kp.m_tiles + 1) / 2 * kp.n_tiles, kp.kb, grid / 2, grid / 2);
   kp.ws = s.ws;
   kp.counters = s.counters;
   kp.err = s.err;

@@ -275,7 +275,7 @@ atspeed_status atspeed_op_gemm_noalloc(atspeed_stream stream, const void* d_W, c
   a.out_f32 = d_Y;
   a.ldo = ldy;
   char eb[256];
-  return gemm_status(gemm_launch(a, s, kNoAllocGrid, (cudaStream_t)stream, false, eb, sizeof eb));
+  return gemm_status(gemm_launch(a, s, kNoAllocGrid, kNoAllocGrid, (cudaStream_t)stream, false, eb, sizeof eb));
 }
 
 /* See include/atspeed.h.  Reads (and clears) the error words that the operators' bounded waits set. */

@@ -238,6 +238,29 @@ def test_full_lse_paths(ats, V, users, N, gamma, d):
     ctx.close()
 
 
+# forwards of more than 256 tokens: split tiles are split for as many CTAs as a 256-token forward has, however
+# many run; 2048 and 4096 tokens of this model (6 to 48 weight tiles, split for 48 CTAs) are whole tiles alone, so
+# a user's logits do not depend on the other users'
+def test_long_forward_sums_do_not_depend_on_the_grid(ats):
+    from types import SimpleNamespace
+    d, f, V, P = 768, 3072, 1024, 1024
+    w = {"embed": _randn((V, d), 1), "lm_head": _randn((V, d), 2, 0.1), "final_norm": _randn((d,), 3, 0.1) + 1}
+    for name, shape in (("attn_norm", (d,)), ("mlp_norm", (d,)), ("wqkv", (3 * d, d)), ("wo", (d, d)),
+                        ("wgate_up", (2 * f, d)), ("wdown", (d, f))):
+        w["layers.0." + name] = _randn(shape, 4 + len(name), 0.02) + (1 if "norm" in name else 0)
+    spec = SimpleNamespace(n_layers=1, d_model=d, n_heads=12, d_ffn=f, vocab=V, rms_eps=1e-6, rope_theta=1e4)
+    items = np.zeros((256, 4), np.int32)
+    items[:, 0] = np.arange(256)
+    tokens = torch.from_numpy(np.random.default_rng(0).integers(0, V, 4 * P).astype(np.int32)).cuda()
+    ctx = ats.Context(spec, w, None, None, items, 0, max_users=4, max_prompt=P, max_K=5, max_N=10, max_gamma=1)
+    got = []
+    for users in (2, 4):
+        ctx.prefill(tokens[:users * P], P * np.arange(users + 1))
+        got.append(ctx.debug_buffer(0, 7, np.float32, 2 * 1024).copy())
+    assert np.array_equal(*got)
+    ctx.close()
+
+
 # the exact selection of a drafted level (score descending, index ascending): one histogram pass, several (an
 # outlier widens the range), none (few candidates), more equal keys than are ranked at once, infinite scores
 @pytest.mark.parametrize("N", [1, 5, 40, 100])
