@@ -66,7 +66,8 @@ def test_gemm_paths(ats, M, K, T):
 
 @pytest.mark.parametrize("F,K,T", [(64, 64, 1), (192, 128, 16), (320, 512, 33), (1408, 1024, 128), (1024, 4096, 130),
                                    (3072, 768, 257), (11008, 256, 250), (9728, 192, 40), (5632, 128, 700),
-                                   (6080, 128, 120), (9792, 128, 70), (960, 512, 400)])
+                                   (6080, 128, 120), (9792, 128, 70), (960, 512, 400),
+                                   (9920, 192, 200), (5632, 2048, 200), (5632, 2048, 90)])
 def test_swiglu_paths(ats, F, K, T):
     W, X = _randn((2 * F, K), F + K, 0.05), _x(T, K, T)
     g, u = (X[:T].double() @ W.double().T).split(F, 1)
@@ -96,6 +97,14 @@ def test_gemm_result_does_not_depend_on_the_token_count(ats, M, K):
     full = ats.op_gemm(W, X, 256)
     for T in (1, 10, 16, 33, 64, 100, 120, 129, 200):
         assert torch.equal(ats.op_gemm(W, X, T), full[:T])
+
+
+@pytest.mark.parametrize("F,K", [(320, 512), (5632, 2048), (11008, 512)])
+def test_swiglu_result_does_not_depend_on_the_token_count(ats, F, K):
+    W, X = _randn((2 * F, K), 5, 0.05), _x(256, K, 6)
+    full = ats.op_gemm_swiglu(W, X, 256)
+    for T in (1, 33, 64, 128, 200):
+        assert torch.equal(ats.op_gemm_swiglu(W, X, T), full[:T])
 
 
 @pytest.mark.parametrize("T,d", [(1, 4), (7, 256), (9, 260), (3, 1024), (17, 1028), (5, 4096), (2, 4100), (3, 8192),
