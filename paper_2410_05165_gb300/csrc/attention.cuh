@@ -39,7 +39,7 @@ struct AttnArgs {
   const int* page_table;           // [users][max_pages] page ids (page p = rows 64p .. 64p+63)
   int max_pages;
   const int* user_splits;          // [users] number of prefix splits of this user
-  int chunks_per_split;            // prefix pages per split (0 = all pages in one split)
+  int chunks_per_split;            // prefix pages per split (0 = all pages in one split; operator: balanced over them)
   int max_splits;                  // grid z
   // outputs
   __nv_bfloat16* out;              // [T][d] attention output (bf16)
